@@ -274,11 +274,6 @@ struct StF32 {
     else
       reinterpret_cast<float*>(b + I.h_off + (size_t)i * I.plane_bytes)[idx] = v;
   }
-  // f_i and g_i of one cell as one 8-byte store
-  __device__ static __forceinline__ void st_fg(const InstDev& I, char* b, int i, size_t idx,
-                                               float fv, float gv) {
-    reinterpret_cast<float2*>(b + (size_t)i * I.pair_bytes)[idx] = make_float2(fv, gv);
-  }
 };
 
 // 16-bit forms: q = s_k v in fp16 / bf16 (v the value or, for hbar, the
@@ -327,24 +322,22 @@ struct StDev {
     }
     put(const_cast<E*>(at(I, b, k, i, idx)), v * I.s[k]);
   }
-  // f_i and g_i (i >= 1) of one cell as one 4-byte store
-  __device__ static __forceinline__ void st_fg(const InstDev& I, char* b, int i, size_t idx,
-                                               float fv, float gv) {
-    put2(reinterpret_cast<E*>(b + (size_t)(i - 1) * I.pair_bytes) + 2 * idx, fv * I.s[0],
-         gv * I.s[1]);
+  // two scaled values as a packed pair, and one, stochastically rounded; the
+  // pair's second value as stored
+  __device__ static __forceinline__ uint32_t sr_pack(float a, float b, uint32_t r) {
+    return BF ? sr_pack_bf162(a, b, r) : sr_pack_half2(a, b, r);
   }
-  // the same, stochastically rounded with the random word r; returns the
-  // stored g_i scaled by s_1 (exact)
-  __device__ static __forceinline__ float st_fg_sr(const InstDev& I, char* b, int i, size_t idx,
-                                                   float fv, float gv, uint32_t r) {
-    const uint32_t q = BF ? sr_pack_bf162(fv * I.s[0], gv * I.s[1], r)
-                          : sr_pack_half2(fv * I.s[0], gv * I.s[1], r);
-    *reinterpret_cast<uint32_t*>(reinterpret_cast<E*>(b + (size_t)(i - 1) * I.pair_bytes) +
-                                 2 * idx) = q;
+  __device__ static __forceinline__ float pack_hi(uint32_t q) {
     if constexpr (BF)
       return __uint_as_float(q & 0xffff0000u);
     else
       return __half2float(__ushort_as_half((unsigned short)(q >> 16)));
+  }
+  __device__ static __forceinline__ E sr_one(float v, uint32_t r) {
+    if constexpr (BF)
+      return sr_bf16(v, r);
+    else
+      return sr_half(v, r);
   }
   // one 16-bit value (not g_0), stochastically rounded
   __device__ static __forceinline__ void st_sr(const InstDev& I, char* b, int k, int i, size_t idx,

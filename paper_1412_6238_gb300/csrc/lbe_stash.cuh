@@ -5,9 +5,17 @@
 // of one instance: a CTA of NC threads marches up the rows, thread t owning
 // column x0 + t.  The stencils also need the moments of the two halo columns
 // on each side (c at x0 - 2 .. x0 + NC + 1, p and T at x0 - 1 .. x0 + NC):
-// four lanes of the last warp form those as extra work, so that no thread
-// of the CTA is spent on a column it does not collide (NC a power of two:
-// the strips tile power-of-two grids exactly).  Instead of staging whole
+// four lanes of a helper warp form those (FP32) or, as extra work, of the
+// last warp, so that no column thread is spent on a column it does not
+// collide (NC a power of two: the strips tile power-of-two grids exactly).
+// The helper warp issues the copies too.  What it is for: on a lone CTA a row
+// took 2,970 cycles, of which warp 0 spent 550 issuing the copies and the
+// last warp 530 on the halo columns, the others waiting at the two barriers
+// for them (clock stamps); with the helper 2,500.  It costs registers: 5
+// warps per CTA leave 128 a thread for 3 CTAs per SM (FP32, which fits since
+// the instance's constants are read from shared memory where they are used)
+// but 96 for 4 (16-bit forms: 612 us a step against 590 without, 4096^2
+// F16MIX, so these have none).  Instead of staging whole
 // source rows (as a TMA tiled row ring would, 7 rows for the pull and the
 // stencils), the CTA stages, for
 // each moment row m, what its cells pull: for each population row of the
@@ -27,16 +35,22 @@
 //   barrier; 1. collide row i-1 (S2-S9 of lbe_cell.cuh) from its stash slot
 //      and the moment rings, and store its 27 values; every thread arrives
 //      on the slot's empty mbarrier right after its pulls;
-//   2. one elected lane of warp 0 waits for that empty barrier and issues
-//      the copies of row i+3 into the slot (as early as possible: the
-//      copies then have the rest of this iteration and the next collision
-//      to land), while the other warps go on;
+//   2. one elected lane (of the helper warp, or of warp 0) waits for that
+//      empty barrier and issues the copies of row i+3 into the slot (as early
+//      as possible: the copies then have the rest of this iteration and the
+//      next collision to land), while the other warps go on;
 //   3. wait for the copies of row i+2 and form its moments c, p, T (S1) into
 //      the rings (own columns, then the four halo columns); rows below the
 //      bottom wall use the pulled values of their mirror row, rows above the
 //      top wall copy the mirror rows in the rings;
 //   barrier; 4. unit normal of row i+1 (S2).
-// Every population is read from HBM once per step.  Every mbarrier wait is
+// Every population is read from HBM once per step.  What bounds it (GB300,
+// 2048^2): FP32 issues 65 % of its slots and moves 79 % of the copy rate's
+// bytes at 4096^2 (665 us a step; 694 before the helper warp, the constants
+// in shared memory, the rings' common row offsets and the stepped store
+// pointers), held by the dependent chain of a row; the 16-bit forms issue 73 %
+// (F16MIX 136 M warp instructions where the address arithmetic of before made
+// it 145 M: 616 -> 590 us at 4096^2, F16DEV 693 -> 672).  Every mbarrier wait is
 // bounded (poll_lim polls): on the first time-out the CTA sets *err, issues
 // no further copy, waits (bounded again) for the copies it has in flight and
 // returns.  A drain wait that also runs out means a copy that was issued has
@@ -115,6 +129,7 @@ struct StashFmt<StF32> {
   static constexpr int LOB = (STASH_NC + 8) * 2;      // its bytes
   static constexpr int SLOT_RAW = LO + LOB;           // bytes of one row
   static constexpr int MINB = 3;                      // resident CTAs per SM
+  static constexpr bool HELPER = true;                // a helper warp
   __host__ __device__ static constexpr int off(int k, int i) {
     return k < 2 ? i * PROW : HOFF + i * ROW;
   }
@@ -137,6 +152,7 @@ struct StashFmt16 {
   static constexpr int LOB = ROW;
   static constexpr int SLOT_RAW = LO + LOB;
   static constexpr int MINB = 4;
+  static constexpr bool HELPER = false;
   __host__ __device__ static constexpr int off(int k, int i) {
     return k == 2 ? HOFF + i * ROW : (i == 0 ? (k == 0 ? F0 : G0) : (i - 1) * PROW);
   }
@@ -155,6 +171,7 @@ struct StashFmt<StMix> {
   static constexpr int G0B = EW * 4;
   static constexpr int SLOT_RAW = G0 + G0B;
   static constexpr int MINB = 4;
+  static constexpr bool HELPER = false;
   static_assert(WROW % 16 == 0 && G0B % 16 == 0, "bulk copies: 16-byte sizes and offsets");
 };
 template <>
@@ -162,7 +179,7 @@ struct StashFmt<StF16> : StashFmt16<__half> {};
 template <>
 struct StashFmt<StBF16> : StashFmt16<__nv_bfloat16> {};
 
-template <class S, int NC>
+template <class S, int NC, bool VAR>
 struct StashCfg {
   using Fmt = StashFmt<S>;
   static_assert(NC == STASH_NC, "the stash formats are laid out for STASH_NC columns");
@@ -174,18 +191,24 @@ struct StashCfg {
   static constexpr int TX = Fmt::SLOT_RAW;    // bytes copied per row
   static constexpr int CR = 5, PR = 5, NR = 4;  // moment / normal ring rows
   static_assert(CR == PR, "c, p and T rings share their row index");
-  // ring row widths: c (and its low part) at x0 - 2 .. x0 + NC + 1, p, T
-  // and the unit normal at x0 - 1 .. x0 + NC
-  static constexpr int CW = NC + 4, QW = NC + 2;
+  // ring row width: c (and its low part) at x0 - 2 .. x0 + NC + 1, and, in
+  // rings of the same width (one row offset serves them all), p, T and the
+  // unit normal at x0 - 1 .. x0 + NC
+  static constexpr int CW = NC + 4;
   static constexpr int STASH = SR * SLOT;
   // FP32 rings of c, p, T, n_x, n_y and the FP16 ring of the c low part
-  static constexpr int RINGS = (CR * CW + 2 * PR * QW + 2 * NR * QW) * 4 + CR * CW * 2;
+  static constexpr int RINGS = (CR + 2 * PR + 2 * NR) * CW * 4 + CR * CW * 2;
   static_assert(RINGS % 8 == 0, "the slot barriers follow the rings");
   // a "full" (copies landed) and an "empty" (every thread done with the
   // slot) mbarrier per stash slot
   static constexpr int SMEM = STASH + RINGS + 2 * SR * 8;
   // resident CTAs per SM the kernel is compiled for (registers)
   static constexpr int MINB = Fmt::MINB;
+  // NC column threads and the helper warp (copies, halo columns).  Not with
+  // the variants (VAR): in FP32 their registers spill at 128 a thread (52
+  // against 45 us a step, 1000 x 777)
+  static constexpr bool HELPER = Fmt::HELPER && !VAR;
+  static constexpr int THREADS = NC + (HELPER ? 32 : 0);
   static_assert(NC % 32 == 0, "whole warps");
 };
 
@@ -554,6 +577,13 @@ __device__ __forceinline__ void issue_row(const CopyPlan& c, uint32_t dst, uint3
   });
 }
 
+// p, stepped to the same cell of the next plane: one 64-bit addition per
+// store (the compiler otherwise forms the 19 plane addresses of a row anew).
+__device__ __forceinline__ void next_plane(char*& p, uint64_t plane) {
+  p += plane;
+  asm volatile("" : "+l"(p));
+}
+
 // VAR: the boundary and property variants (harmonic law, wall temperature
 // at the link's wall crossing, wetting walls) compiled in; without them the
 // kernel carries none of their registers.
@@ -561,34 +591,40 @@ __device__ __forceinline__ void issue_row(const CopyPlan& c, uint32_t dst, uint3
 // (a compile-time choice: compiled in, the ghost stores cost the main
 // stores about 1 % even where no lane takes them).
 template <class S, int NC, bool VAR, bool OWN>
-__global__ void __launch_bounds__(NC, (StashCfg<S, NC>::MINB))
+__global__ void __launch_bounds__(StashCfg<S, NC, VAR>::THREADS, (StashCfg<S, NC, VAR>::MINB))
 stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items, int seg_rows,
              int parity, int* __restrict__ err, int poll_lim, int withhold,
              const uint32_t* __restrict__ seed) {
-  using Cfg = StashCfg<S, NC>;
+  using Cfg = StashCfg<S, NC, VAR>;
   using Fmt = typename Cfg::Fmt;
   using C = float;
   constexpr bool W16 = sizeof(typename Fmt::E) == 2;
   constexpr bool MIX = S::kind == ST_F16MIX;
   extern __shared__ __align__(128) char smem[];
-  constexpr int CW = Cfg::CW, QW = Cfg::QW;
-  // ring entry of column x0 + j: c (and its low part) at j + 2, p, T, n at j + 1
+  constexpr int CW = Cfg::CW;
+  // ring entry of column x0 + j: j + 2
   C* cring = reinterpret_cast<C*>(smem + Cfg::STASH);  // [CR][CW]
-  C* pring = cring + Cfg::CR * CW;                       // [PR][QW]
-  C* Tring = pring + Cfg::PR * QW;                       // [PR][QW]
-  C* nxr = Tring + Cfg::PR * QW;                         // [NR][QW]
-  C* nyr = nxr + Cfg::NR * QW;
-  __half* clr = reinterpret_cast<__half*>(nyr + Cfg::NR * QW);  // [CR][CW], lo * 2^24
+  C* pring = cring + Cfg::CR * CW;                       // [PR][CW]
+  C* Tring = pring + Cfg::PR * CW;                       // [PR][CW]
+  C* nxr = Tring + Cfg::PR * CW;                         // [NR][CW]
+  C* nyr = nxr + Cfg::NR * CW;
+  __half* clr = reinterpret_cast<__half*>(nyr + Cfg::NR * CW);  // [CR][CW], lo * 2^24
   // [SR] full barriers, then [SR] empty barriers
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::STASH + Cfg::RINGS);
   __shared__ int s_abort;
+  __shared__ __align__(16) Phys<C> s_phys;  // the item's constants
   const int t = threadIdx.x;
   const int wu = __shfl_sync(0xffffffffu, t >> 5, 0);  // the warp index, warp-uniform
-  // halo lanes: lanes 0..3 of the last warp form the moments of columns
-  // x0 - 2, x0 - 1, x0 + NC, x0 + NC + 1 (offset hj from x0)
+  // The halo columns x0 - 2, x0 - 1, x0 + NC, x0 + NC + 1 (offset hj from x0)
+  // are formed by lanes 0..3 of a helper warp, which issues the copies too
+  // (HELPER), or, after their own column, of the last warp.  The threads of
+  // the other warps own column x0 + t.
+  constexpr bool HELPER = Cfg::HELPER;
+  const bool helper = HELPER && wu == Cfg::NW;
   const int lane = t & 31;
-  const bool halo = wu == Cfg::NW - 1 && lane < 4;
   const int hj = lane < 2 ? lane - 2 : NC - 2 + lane;
+  const bool halo = wu == (HELPER ? Cfg::NW : Cfg::NW - 1) && lane < 4;
+  const int own = helper ? hj : t;  // the thread's column, from x0
   const uint32_t stash_u = smem_u32(smem);
   const uint32_t bars_u = smem_u32(bars);
   const uint32_t empty_u = bars_u + 8 * Cfg::SR;
@@ -666,18 +702,22 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
     ya = __shfl_sync(0xffffffffu, ya, 0);
     yb = __shfl_sync(0xffffffffu, yb, 0);
     char* __restrict__ dst = I.buf[parity ^ 1];
-    Phys<C> P = phys<C>(I);
-    if constexpr (!VAR) {  // the variants are off: known to the compiler
-      P.harm = C(0);
-      P.wmid = C(0);
-      P.kw = C(0);
-    }
-    const C en2 = P.eta_n2;
+    // the instance's constants, from shared memory where they are used (held
+    // in registers over the row loop they made the loop spill)
+    auto params = [&]() {
+      Phys<C> P = s_phys;
+      if constexpr (!VAR) {  // the variants are off: known to the compiler
+        P.harm = C(0);
+        P.wmid = C(0);
+        P.kw = C(0);
+      }
+      return P;
+    };
     const uint32_t skey = S::SR ? sr_step_key(step, I.salt) : 0u;
     const size_t pitch = (size_t)I.pitch;
-    const int x = x0 + t;
+    const int x = x0 + own;
     const int xw = wrapx(x, nx);
-    const bool collides = x < nx;
+    const bool collides = !helper && x < nx;
     // OWN: the periodic ghost copies are written by the owner of the cell,
     // element XG + x + nx for x < XG (right ghosts), XG + x - nx for
     // x >= nx - XG (left ghosts), both for 4 <= nx < 2 XG; otherwise
@@ -690,22 +730,23 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
     // which starts at element x0 (a multiple of NC: 16-byte aligned).
     const int e16 = x0 & ~7;
     static_assert(XG == 4, "stash columns: column x0 + j at element j + 4 of a row");
-    const int c0 = (W16 ? x0 - e16 : 0) + t + XG;  // own column in a population row
-    const int c0g = t + XG;                         // own column in the FP32 g_0 row
-    const int c0lo = x0 - e16 + t + XG;             // own column in the g_0 low-part row
-    const int hd = hj - t;                          // halo lanes: column offset from own
-    const int hxw = wrapx(x0 + hj, nx);
+    const int c0 = (W16 ? x0 - e16 : 0) + own + XG;  // own column in a population row
+    const int c0g = own + XG;                         // own column in the FP32 g_0 row
+    const int c0lo = x0 - e16 + own + XG;             // own column in the g_0 low-part row
     const CopyPlan cp = copy_plan(I, parity, x0);
     __syncthreads();  // the previous item is done with the rings and stashes
     if (t == 0) s_abort = 0;
+    constexpr int NP = sizeof(Phys<C>) / sizeof(C);
+    static_assert(NP <= NC, "one constant per thread");
+    if (t < NP) reinterpret_cast<C*>(&s_phys)[t] = reinterpret_cast<const C*>(&phys<C>(I))[t];
 
     auto slot = [&](int m) { return smem + (m & (Cfg::SR - 1)) * Cfg::SLOT; };
     auto rrow = [](int m) { return ((m % Cfg::CR) + Cfg::CR) % Cfg::CR; };
-    auto nr = [](int m) { return (m & (Cfg::NR - 1)) * QW; };
+    auto nr = [](int m) { return (m & (Cfg::NR - 1)) * CW; };
     auto loadable = [&](int m) { return m <= yb + 1 && m < ny; };
     // the copies of the populations pulled by moment row m (the mirror row's
-    // below the bottom wall), issued by one elected lane of warp 0.  In the
-    // row loop the slot is that of the row collided in the same iteration:
+    // below the bottom wall), issued by one elected lane of the helper
+    // warp (or warp 0).  In the row loop the slot is that of the row collided in the same iteration:
     // the lane first waits (bounded) for the slot's empty barrier, on which
     // every thread arrives once per iteration after its last read of the
     // slot (release = false: the slot is free already, at an item start).
@@ -715,7 +756,7 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
       if (release) ephase ^= 1u << sl;  // one release of this slot per iteration
       if (!loadable(m)) return;
       pending |= 1u << sl;
-      if (wu != 0) return;
+      if (HELPER ? !helper : wu != 0) return;
       __syncwarp();
       if (elect_one()) {
         if (release && !mbar_wait(empty_u + 8 * sl, epar, poll_lim)) {
@@ -749,13 +790,18 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
     };
 
     issue(ya - 2, false);
-    int i5 = (((ya - 4) % Cfg::CR) + Cfg::CR) % Cfg::CR;  // i mod CR
-    for (int i = ya - 4; i <= yb; i++, i5 = (i5 == Cfg::CR - 1) ? 0 : i5 + 1) {
-      // ring row of i + d (|d| < CR)
-      auto rr = [&](int d) {
-        int v = i5 + d;
-        return v < 0 ? v + Cfg::CR : (v >= Cfg::CR ? v - Cfg::CR : v);
-      };
+    // ring offsets of rows i - 2 .. i + 2, rotated from row to row
+    int om2 = rrow(ya - 6) * CW, om1 = rrow(ya - 5) * CW, o0 = rrow(ya - 4) * CW;
+    int o1 = rrow(ya - 3) * CW, o2 = rrow(ya - 2) * CW;
+    auto rotate = [&]() {
+      const int f = om2;
+      om2 = om1;
+      om1 = o0;
+      o0 = o1;
+      o1 = o2;
+      o2 = f;
+    };
+    for (int i = ya - 4; i <= yb; i++, rotate()) {
       __syncthreads();
       if (s_abort) break;
 
@@ -765,6 +811,7 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
       if (r >= ya && r < yb && collides) {
         const char* s = slot(r);
         C f[9], g[9], h[9], g0lo;
+        const Phys<C> P = params();
         // hbar as pulled (without the change of reference row in interior
         // rows, which collide() applies through the source term)
         if constexpr (MIX) {
@@ -779,19 +826,18 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
           g0lo = __half2float(reinterpret_cast<const __half*>(s + Fmt::LO)[c0lo]) * G0LO_INV;
         }
         mbar_arrive(ebar);  // done with the slot (the arrive orders the reads before it)
-        const int ps = rr(-2), p0 = rr(-1), pn = rr(0);  // rows r-1, r, r+1
-        // rows of the rings from column x0 (index t: the own column)
-        const C* cs = cring + ps * CW + 2;
-        const C* c0 = cring + p0 * CW + 2;
-        const C* cn = cring + pn * CW + 2;
+        // rows r - 1, r, r + 1 of the rings from column x0 (index t: own)
+        const C* cs = cring + om2 + 2;
+        const C* c0 = cring + om1 + 2;
+        const C* cn = cring + o0 + 2;
         const C cc = c0[t];
-        const C clo = lo_at(clr + p0 * CW + 2, t);
-        const C* Ts = Tring + ps * QW + 1;
-        const C* T0 = Tring + p0 * QW + 1;
-        const C* Tn = Tring + pn * QW + 1;
-        const C* qs = pring + ps * QW + 1;
-        const C* q0 = pring + p0 * QW + 1;
-        const C* qn = pring + pn * QW + 1;
+        const C clo = lo_at(clr + om1 + 2, t);
+        const C* Ts = Tring + om2 + 2;
+        const C* T0 = Tring + om1 + 2;
+        const C* Tn = Tring + o0 + 2;
+        const C* qs = pring + om2 + 2;
+        const C* q0 = pring + om1 + 2;
+        const C* qn = pring + o0 + 2;
         const C pp = q0[t], TT = T0[t];
         Stencils<C> st;
         grad3(cs, c0, cn, t, st.gcx, st.gcy);
@@ -799,7 +845,7 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
         grad3(Ts, T0, Tn, t, st.gTx, st.gTy);
         if (dev_h<S>()) st.gTy += P.hr1;
         grad3(qs, q0, qn, t, st.gpx, st.gpy);
-        const int ns = nr(r - 1) + 1, n0 = nr(r) + 1, nn = nr(r + 1) + 1;
+        const int ns = nr(r - 1) + 2, n0 = nr(r) + 2, nn = nr(r + 1) + 2;
         C d1, d2, dum;
         grad3(nxr + ns, nxr + n0, nxr + nn, t, d1, dum);
         grad3(nyr + ns, nyr + n0, nyr + nn, t, dum, d2);
@@ -819,43 +865,61 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
           if constexpr (MIX) {
             // word i: (f_i, g_i, hbar_i); word 0: (f_0, hbar_0, g_0 low part)
             const float s1 = I.s[1], s2 = I.s[2];
-            auto word = [&](int ii, float fv, uint32_t u) {
-              reinterpret_cast<uint2*>(dst + (size_t)ii * I.pair_bytes)[e] =
-                  make_uint2(__float_as_uint(fv), u);
-            };
             float gs = 0.f;  // the stored g_i, times s_1
+            char* const w0 = dst + 8 * e;
+            char* w = w0;
 #pragma unroll
             for (int ii = 1; ii < 9; ii++) {
               const uint32_t q =
                   sr_pack_half2(o[9 + ii] * s1, o[18 + ii] * s2, S::sr_word(1, ii, hc));
               gs += __half2float(__ushort_as_half((unsigned short)(q & 0xffffu)));
-              word(ii, o[ii], q);
+              next_plane(w, I.pair_bytes);
+              *reinterpret_cast<uint2*>(w) = make_uint2(__float_as_uint(o[ii]), q);
             }
             float g0h, g0l;
             g0_remainder(cc, clo, gs * P.inv_s[1], g0h, g0l);
-            word(0, o[0],
-                 (uint32_t)__half_as_ushort(sr_half(o[18] * s2, S::sr_word(2, 0, hc))) |
-                     ((uint32_t)__half_as_ushort(__float2half_rn(g0l * G0LO_SCALE)) << 16));
+            *reinterpret_cast<uint2*>(w0) = make_uint2(
+                __float_as_uint(o[0]),
+                (uint32_t)__half_as_ushort(sr_half(o[18] * s2, S::sr_word(2, 0, hc))) |
+                    ((uint32_t)__half_as_ushort(__float2half_rn(g0l * G0LO_SCALE)) << 16));
             reinterpret_cast<float*>(dst + I.g0_off)[e] = g0h;
           } else if constexpr (!W16) {
             st_g0lo<S>(I, dst, e, lo_out);
+            char* w = dst + 8 * e;
 #pragma unroll
-            for (int ii = 0; ii < 9; ii++) S::st_fg(I, dst, ii, e, o[ii], o[9 + ii]);
+            for (int ii = 0; ii < 9; ii++) {
+              *reinterpret_cast<float2*>(w) = make_float2(o[ii], o[9 + ii]);
+              next_plane(w, I.pair_bytes);
+            }
+            w = dst + I.h_off + 4 * e;
 #pragma unroll
-            for (int ii = 0; ii < 9; ii++) S::st(I, dst, 2, ii, e, o[18 + ii]);
+            for (int ii = 0; ii < 9; ii++) {
+              *reinterpret_cast<float*>(w) = o[18 + ii];
+              next_plane(w, I.plane_bytes);
+            }
           } else {
             S::st_sr(I, dst, 0, 0, e, o[0], S::sr_word(0, 0, hc));
             float gs = 0.f;  // the stored g_i, times s_1
+            const float s0 = I.s[0], s1 = I.s[1], s2 = I.s[2];
+            char* w = dst + 4 * e;
 #pragma unroll
-            for (int ii = 1; ii < 9; ii++)
-              gs += S::st_fg_sr(I, dst, ii, e, o[ii], o[9 + ii], S::sr_word(0, ii, hc));
+            for (int ii = 1; ii < 9; ii++) {
+              const uint32_t q = S::sr_pack(o[ii] * s0, o[9 + ii] * s1, S::sr_word(0, ii, hc));
+              gs += S::pack_hi(q);
+              *reinterpret_cast<uint32_t*>(w) = q;
+              next_plane(w, I.pair_bytes);
+            }
             float g0h, g0l;
             g0_remainder(cc, clo, gs * P.inv_s[1], g0h, g0l);
             S::st(I, dst, 1, 0, e, g0h);
             st_g0lo<S>(I, dst, e, g0l);
+            w = dst + I.h_off + 2 * e;
 #pragma unroll
-            for (int ii = 0; ii < 9; ii++)
-              S::st_sr(I, dst, 2, ii, e, o[18 + ii], S::sr_word(2, ii, hc));
+            for (int ii = 0; ii < 9; ii++) {
+              *reinterpret_cast<typename Fmt::E*>(w) =
+                  S::sr_one(o[18 + ii] * s2, S::sr_word(2, ii, hc));
+              next_plane(w, I.plane_bytes);
+            }
           }
         };
         store_at((size_t)r * pitch + XG + x);
@@ -866,7 +930,7 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
               store_at((size_t)r * pitch + (XG + x + ((dq == 1 && gR) ? nx : -nx)));
           }
         }
-      } else {
+      } else if (!helper) {
         mbar_arrive(ebar);
       }
 
@@ -883,10 +947,10 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
         atomicOr(err, 1);
       }
       if (m <= yb + 1) {
-        const int rm = rr(2);
         // moments of the column at offset dj from the own one into ring
-        // entries ci (c) and, if pt, pi (p, T)
-        auto moments = [&](int dj, int cxw, int ci, int pi, bool pt) {
+        // entry ci of c and, if pt, of p and T
+        auto moments = [&](int dj, int cxw, int ci, bool pt) {
+          const Phys<C> P = params();
           if (m < ny) {
             const int mr = m >= 0 ? m : -1 - m;
             const char* s = slot(m);
@@ -907,8 +971,8 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
                 cring[ci] = m < 0 ? wet_ghost(P, cv, -1 - m) : cv;
                 clr[ci] = __float2half_rn(clo * G0LO_SCALE);
                 if (pt) {
-                  pring[pi] = pv;
-                  Tring[pi] = m < 0 ? ghost_T<S>(I, cxw, true, Tv) : Tv;
+                  pring[ci] = pv;
+                  Tring[ci] = m < 0 ? ghost_T<S>(I, cxw, true, Tv) : Tv;
                 }
                 done = true;
               }
@@ -921,10 +985,10 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
               if (m < 0) cring[ci] = wet_ghost(P, cring[ci], -1 - m);
               clr[ci] = __float2half_rn(clo * G0LO_SCALE);
               if (pt) {
-                pring[pi] = sum9(vf);
+                pring[ci] = sum9(vf);
                 C T = dv(sum9(vh), P.rho_cv, P.inv_rho_cv);
                 if (m < 0) T = ghost_T<S>(I, cxw, true, T);
-                Tring[pi] = T;
+                Tring[ci] = T;
               }
             } else {
               if constexpr (!W16) {
@@ -940,29 +1004,27 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
               if (m < 0) cring[ci] = wet_ghost(P, cring[ci], -1 - m);
               clr[ci] = __float2half_rn(clo * G0LO_SCALE);
               if (pt) {
-                pring[pi] = sum9(vf);
+                pring[ci] = sum9(vf);
                 wstash_pull<S, 2, true>(I, P, s, c0 + dj, c0g + dj, mr, cxw, v);
                 C T = dv(sum9(v), P.rho_cv, P.inv_rho_cv);
                 if (m < 0) T = ghost_T<S>(I, cxw, true, T);
-                Tring[pi] = T;
+                Tring[ci] = T;
               }
             }
           } else {
             // above the top wall: the mirror row's moments
-            const int mm = rrow(2 * ny - 1 - m);
-            const int cm = ci - rm * CW + mm * CW, pm = pi - rm * QW + mm * QW;
+            const int cm = ci - o2 + rrow(2 * ny - 1 - m) * CW;
             cring[ci] = wet_ghost(P, cring[cm], m - ny);
             clr[ci] = clr[cm];
             if (pt) {
-              pring[pi] = pring[pm];
-              Tring[pi] = ghost_T<S>(I, cxw, false, Tring[pm]);
+              pring[ci] = pring[cm];
+              Tring[ci] = ghost_T<S>(I, cxw, false, Tring[cm]);
             }
           }
         };
-        moments(0, xw, rm * CW + t + 2, rm * QW + t + 1, true);
+        if (!helper) moments(0, xw, o2 + t + 2, true);
         // the halo columns: c of all four, p and T of x0 - 1 and x0 + NC
-        if (halo)
-          moments(hd, hxw, rm * CW + hj + 2, rm * QW + hj + 1, lane == 1 || lane == 2);
+        if (halo) moments(hj - own, wrapx(x0 + hj, nx), o2 + hj + 2, lane == 1 || lane == 2);
       }
       __syncthreads();
       if (s_abort) break;
@@ -970,13 +1032,15 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
       // ---- 4. unit normal of row i + 1
       const int mn = i + 1;
       if (mn >= ya - 1 && mn <= yb) {
-        const C* ca = cring + rr(0) * CW;
-        const C* cb = cring + rr(1) * CW;
-        const C* cc2 = cring + rr(2) * CW;
-        normal3(ca, cb, cc2, t + 2, en2, nxr[nr(mn) + t + 1], nyr[nr(mn) + t + 1]);
+        const C* ca = cring + o0;
+        const C* cb = cring + o1;
+        const C* cc2 = cring + o2;
+        auto normal = [&](int j) {
+          normal3(ca, cb, cc2, j + 2, s_phys.eta_n2, nxr[nr(mn) + j + 2], nyr[nr(mn) + j + 2]);
+        };
+        if (!helper) normal(t);
         // the halo columns x0 - 1 and x0 + NC
-        if (halo && (lane == 1 || lane == 2))
-          normal3(ca, cb, cc2, hj + 2, en2, nxr[nr(mn) + hj + 1], nyr[nr(mn) + hj + 1]);
+        if (halo && (lane == 1 || lane == 2)) normal(hj);
       }
     }
     __syncthreads();

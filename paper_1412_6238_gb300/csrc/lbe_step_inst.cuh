@@ -89,7 +89,7 @@ bool stash_attr() {
   if (!done[dev]) {
     if (cudaFuncSetAttribute(stash_kernel<LBE_ST, NC, VAR, OWN>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             StashCfg<LBE_ST, NC>::SMEM) != cudaSuccess)
+                             StashCfg<LBE_ST, NC, VAR>::SMEM) != cudaSuccess)
       return false;
     done[dev] = true;
   }
@@ -103,16 +103,17 @@ cudaError_t stash_one(const InstDev* d, int n, int64_t items, int seg, int parit
   if (grid <= 0) grid = 1;
   if ((int64_t)grid > items) grid = (int)items;
   stash_kernel<LBE_ST, NC, VAR, OWN>
-      <<<grid, NC, StashCfg<LBE_ST, NC>::SMEM, s>>>(d, n, items, seg, parity, err, poll_lim,
-                                                    withhold, seed);
+      <<<grid, StashCfg<LBE_ST, NC, VAR>::THREADS, StashCfg<LBE_ST, NC, VAR>::SMEM, s>>>(
+          d, n, items, seg, parity, err, poll_lim, withhold, seed);
   return cudaGetLastError();
 }
 template <int NC, bool VAR, bool OWN>
 int stash_occ() {
   if (!stash_attr<NC, VAR, OWN>()) return 0;
   int b = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, stash_kernel<LBE_ST, NC, VAR, OWN>, NC,
-                                                    StashCfg<LBE_ST, NC>::SMEM) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, stash_kernel<LBE_ST, NC, VAR, OWN>,
+                                                    StashCfg<LBE_ST, NC, VAR>::THREADS,
+                                                    StashCfg<LBE_ST, NC, VAR>::SMEM) != cudaSuccess)
     return 0;
   return b;
 }
