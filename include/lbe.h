@@ -263,15 +263,16 @@ typedef struct {
   int64_t window;      /* 1 <= W <= N: states averaged into the loss          */
   int64_t ckpt_every;  /* k >= 1: spacing of the stored checkpoints; the
                           backward recomputes each segment of k steps from
-                          its checkpoint and keeps k + 1 FP64 states          */
+                          its checkpoint and keeps k + 1 states               */
 } lbe_adjoint_spec;
 
 /* Forward N steps from the handle's current state (the handle's storage and
  * kernel; checkpoints of the raw storage every k steps), then the backward
- * sweep over the recomputed states (kept as FP64).  The backward arithmetic
- * follows the forward's: FP64 for an LBE_F64 handle; FP32 per-cell products
- * for the other storages, whose trajectory is an FP32 one (the adjoint
- * vectors and the parameter sums stay FP64; the loss is always FP64).
+ * sweep over the recomputed states.  The backward arithmetic follows the
+ * forward's: FP64 for an LBE_F64 handle; FP32 per-cell products for the other
+ * storages, whose trajectory is an FP32 one (an adjoint is then held as the
+ * two FP32 parts whose sum it is; the parameter sums stay FP64, the loss is
+ * always FP64).
  * Outputs (each may be NULL):
  *   loss     host double: L
  *   grad     host double[3]: dL/dsigmaT, dL/d(eta2/eta1), dL/d(lam2/lam1)
@@ -280,7 +281,8 @@ typedef struct {
  * dT0 and dQ0 are device pointers if on_device, else host.  The handle must
  * hold one instance.  On return the handle holds the state after the N steps
  * (steps_done advanced by N).  Device memory used during the call:
- * about (k + 1 + 2) * 27 + 30 doubles per cell plus N/k raw checkpoints; it is
+ * about 32 (k + 1) + 71 values per cell (doubles for an LBE_F64 handle, floats
+ * otherwise) plus N/k raw checkpoints; it is
  * allocated and freed inside the call (LBE_ENOMEM if it does not fit).
  * Waits. */
 lbe_status lbe_adjoint(lbe_handle* h, const lbe_adjoint_spec* spec, double* loss,

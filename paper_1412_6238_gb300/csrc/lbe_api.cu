@@ -822,17 +822,27 @@ lbe_status adjoint_run(lbe_handle* h, const lbe_adjoint_spec& sp, double* loss, 
   // handle, FP32 otherwise (the trajectory is then an FP32 one anyway)
   const bool fp32 = h->storage != LBE_F64;
   lbe_status st;
+  const size_t rb = adjoint_real_bytes(fp32);
+  const size_t state_b = rb * (size_t)adjoint_state_planes(fp32) * N;
+  const size_t vec_b = rb * (size_t)adjoint_vector_planes() * N;
+  const size_t part_b = sizeof(double) * (size_t)adjoint_part_doubles(nx, ny);
   DevBuf ck, states, abuf, scr, small, fin;
   if ((st = dalloc(h, ck, (size_t)nseg * H.buf_bytes, "checkpoints"))) return st;
-  if ((st = dalloc(h, states, sizeof(double) * (size_t)(kk + 1) * S27, "segment states"))) return st;
-  if ((st = dalloc(h, abuf, sizeof(double) * 2 * S27, "adjoint states"))) return st;
-  if ((st = dalloc(h, scr, sizeof(double) * (size_t)adjoint_scratch_doubles(nx, ny), "scratch")))
+  if ((st = dalloc(h, states, (size_t)(kk + 1) * state_b, "segment states"))) return st;
+  if ((st = dalloc(h, abuf, 2 * vec_b, "adjoint states"))) return st;
+  // scratch planes; at the end of the sweep the FP64 results for a host copy
+  const size_t host_b = on_device ? 0 : sizeof(double) * (dQ0 ? S27 : dT0 ? N : 0);
+  if ((st = dalloc(h, scr, std::max(rb * (size_t)adjoint_scratch_planes() * N, host_b), "scratch")))
     return st;
-  if ((st = dalloc(h, small, sizeof(double) * (size_t)(4 + 4 * W), "reductions"))) return st;
+  // theta sums, observables of the window, partial sums of each
+  if ((st = dalloc(h, small, sizeof(double) * (size_t)(4 + 4 * W) + 2 * part_b, "reductions")))
+    return st;
   if ((st = dalloc(h, fin, H.buf_bytes, "final state"))) return st;
   double* theta = small.d();
   double* obs = theta + 4;
-  CU(h, cudaMemsetAsync(theta, 0, sizeof(double) * 4, h->stream));
+  double* tpart = obs + 4 * W;
+  double* opart = tpart + part_b / sizeof(double);
+  CU(h, cudaMemsetAsync(tpart, 0, part_b, h->stream));
   auto cur_buf = [&]() { return H.arena + (size_t)h->parity * H.buf_bytes; };
 
   // forward: raw checkpoint at the start of every segment
@@ -848,8 +858,9 @@ lbe_status adjoint_run(lbe_handle* h, const lbe_adjoint_spec& sp, double* loss, 
   CU(h, cudaMemcpyAsync(fin.p, cur_buf(), H.buf_bytes, cudaMemcpyDeviceToDevice, h->stream));
 
   // reverse sweep over the segments; a_nxt holds dL/dQ_{n+1}
-  double* a_cur = abuf.d();
-  double* a_nxt = abuf.d() + S27;
+  char* a_cur = abuf.p;
+  char* a_nxt = abuf.p + vec_b;
+  auto terms = [&](char* v) { return v + rb * S27; };  // an adjoint's terms of the cell
   bool have_next = false;
   const int64_t first_w = NS - W + 1;
   for (int64_t sg = nseg - 1; sg >= 0; sg--) {
@@ -860,19 +871,23 @@ lbe_status adjoint_run(lbe_handle* h, const lbe_adjoint_spec& sp, double* loss, 
     // the step counter as in the forward run, so that the stochastic
     // rounding of a 16-bit storage recomputes the same states
     CU(h, launch_seed_set(h->d_seed, (uint32_t)(steps0 + n0), h->stream));
-    cudaError_t e = launch_pull(h->storage, d1, nx, ny, states.d(), h->parity, h->stream);
+    cudaError_t e =
+        launch_adjoint_state(h->storage, d1, nx, ny, h->parity, states.p, h->stream);
     for (int64_t t = 1; e == cudaSuccess && t <= n1 - n0; t++) {
       if ((st = launch_steps_direct(h, 1))) return st;
-      e = launch_pull(h->storage, d1, nx, ny, states.d() + (size_t)t * S27, h->parity, h->stream);
+      e = launch_adjoint_state(h->storage, d1, nx, ny, h->parity, states.p + (size_t)t * state_b,
+                               h->stream);
     }
     for (int64_t n = n1; e == cudaSuccess && n >= n0; n--) {
-      const double* Q = states.d() + (size_t)(n - n0) * S27;
+      const char* Q = states.p + (size_t)(n - n0) * state_b;
+      const char* cpt = Q + rb * S27;
       const double wl = n >= first_w ? 1.0 / (double)W : 0.0;
       double* o = n >= first_w ? obs + 4 * (n - first_w) : nullptr;
-      if (o) e = launch_observable(d1, nx, ny, Q, scr.d(), o, h->stream);
+      if (o) e = launch_observable(d1, nx, ny, fp32, Q, cpt, opart, o, h->stream);
       if (e == cudaSuccess)
-        e = launch_adjoint_step(d1, nx, ny, Q, have_next ? a_nxt : nullptr, wl, o, a_cur, theta,
-                                scr.d(), fp32, h->stream);
+        e = launch_adjoint_step(d1, nx, ny, fp32, Q, cpt, have_next ? a_nxt : nullptr,
+                                have_next ? terms(a_nxt) : nullptr, wl, o, a_cur, terms(a_cur),
+                                scr.p, tpart, h->stream);
       std::swap(a_cur, a_nxt);
       have_next = true;
     }
@@ -880,18 +895,18 @@ lbe_status adjoint_run(lbe_handle* h, const lbe_adjoint_spec& sp, double* loss, 
     if ((st = wait(h))) return st;
   }
   // a_nxt = dL/dQ_0
+  CU(h, launch_adjoint_sums(tpart, nx, ny, theta, h->stream));
   if (dT0) {
     double* dst = on_device ? dT0 : scr.d();
-    cudaError_t e = launch_adjoint_dT0(d1, nx, ny, a_nxt, dst, h->stream);
+    cudaError_t e = launch_adjoint_dT0(d1, nx, ny, fp32, a_nxt, terms(a_nxt), dst, h->stream);
     if (e != cudaSuccess) return fail(h, LBE_ECUDA, "dT0 kernel: %s", cudaGetErrorString(e));
     if (!on_device && (st = to_host(h, dT0, dst, sizeof(double) * N))) return st;
   }
   if (dQ0) {
-    if (on_device)
-      CU(h, cudaMemcpyAsync(dQ0, a_nxt, sizeof(double) * S27, cudaMemcpyDeviceToDevice,
-                            h->stream));
-    else if ((st = to_host(h, dQ0, a_nxt, sizeof(double) * S27)))
-      return st;
+    double* dst = on_device ? dQ0 : scr.d();
+    cudaError_t e = launch_adjoint_finish(nx, ny, fp32, a_nxt, terms(a_nxt), dst, h->stream);
+    if (e != cudaSuccess) return fail(h, LBE_ECUDA, "dQ0 kernel: %s", cudaGetErrorString(e));
+    if (!on_device && (st = to_host(h, dQ0, dst, sizeof(double) * S27))) return st;
   }
   std::vector<double> hobs(4 * (size_t)W), hth(4);
   if ((st = to_host(h, hobs.data(), obs, sizeof(double) * 4 * W))) return st;
@@ -1212,18 +1227,29 @@ lbe_status lbe_adjoint_step(lbe_handle* h, const double* Q, const double* a_next
   if (st) return st;
   if (!Q || !a_out) return fail(h, LBE_EINVAL, "Q and a_out must be device pointers");
   const InstHost& H = h->inst[0];
+  const size_t N = (size_t)H.nx * H.ny, np = (size_t)adjoint_part_doubles(H.nx, H.ny);
+  // c, p, T; the adjoint; scratch
+  const size_t nv = (size_t)adjoint_vector_planes();
   DevBuf scr, small;
-  if ((st = dalloc(h, scr, sizeof(double) * (size_t)adjoint_scratch_doubles(H.nx, H.ny), "scratch")))
+  if ((st = dalloc(h, scr, sizeof(double) * (3 + nv + (size_t)adjoint_scratch_planes()) * N,
+                   "scratch")))
     return st;
-  if ((st = dalloc(h, small, sizeof(double) * 8, "reductions"))) return st;
+  if ((st = dalloc(h, small, sizeof(double) * (8 + 2 * np), "reductions"))) return st;
+  double* cpt = scr.d();
+  double* av = cpt + 3 * N;
   double* theta = small.d();
   double* obs = theta + 4;
-  CU(h, cudaMemsetAsync(theta, 0, sizeof(double) * 4, h->stream));
-  cudaError_t e = cudaSuccess;
-  if (wl != 0.0) e = launch_observable(h->d_finst, H.nx, H.ny, Q, scr.d(), obs, h->stream);
+  double* tpart = obs + 4;
+  CU(h, cudaMemsetAsync(tpart, 0, sizeof(double) * np, h->stream));
+  cudaError_t e = launch_adjoint_moments(h->d_finst, H.nx, H.ny, Q, cpt, h->stream);
+  if (e == cudaSuccess && wl != 0.0)
+    e = launch_observable(h->d_finst, H.nx, H.ny, false, Q, cpt, tpart + np, obs, h->stream);
   if (e == cudaSuccess)
-    e = launch_adjoint_step(h->d_finst, H.nx, H.ny, Q, a_next, wl, obs, a_out, theta, scr.d(),
-                            false, h->stream);
+    e = launch_adjoint_step(h->d_finst, H.nx, H.ny, false, Q, cpt, a_next, nullptr, wl, obs, av,
+                            av + 27 * N, av + nv * N, tpart, h->stream);
+  if (e == cudaSuccess) e = launch_adjoint_sums(tpart, H.nx, H.ny, theta, h->stream);
+  if (e == cudaSuccess)
+    e = launch_adjoint_finish(H.nx, H.ny, false, av, av + 27 * N, a_out, h->stream);
   if (e != cudaSuccess) return fail(h, LBE_ECUDA, "adjoint step: %s", cudaGetErrorString(e));
   double th[4];
   if ((st = to_host(h, th, theta, sizeof th))) return st;
@@ -1238,11 +1264,14 @@ lbe_status lbe_observable(lbe_handle* h, const double* Q, double* out) {
   if (st) return st;
   if (!Q || !out) return fail(h, LBE_EINVAL, "Q (device) and out (host) must not be NULL");
   const InstHost& H = h->inst[0];
+  const size_t N = (size_t)H.nx * H.ny, np = (size_t)adjoint_part_doubles(H.nx, H.ny);
   DevBuf scr, small;
-  if ((st = dalloc(h, scr, sizeof(double) * (size_t)adjoint_scratch_doubles(H.nx, H.ny), "scratch")))
-    return st;
-  if ((st = dalloc(h, small, sizeof(double) * 4, "reductions"))) return st;
-  cudaError_t e = launch_observable(h->d_finst, H.nx, H.ny, Q, scr.d(), small.d(), h->stream);
+  if ((st = dalloc(h, scr, sizeof(double) * 3 * N, "scratch"))) return st;
+  if ((st = dalloc(h, small, sizeof(double) * (4 + np), "reductions"))) return st;
+  cudaError_t e = launch_adjoint_moments(h->d_finst, H.nx, H.ny, Q, scr.d(), h->stream);
+  if (e == cudaSuccess)
+    e = launch_observable(h->d_finst, H.nx, H.ny, false, Q, scr.d(), small.d() + 4, small.d(),
+                          h->stream);
   if (e != cudaSuccess) return fail(h, LBE_ECUDA, "observable: %s", cudaGetErrorString(e));
   double o[4];
   if ((st = to_host(h, o, small.d(), sizeof o))) return st;

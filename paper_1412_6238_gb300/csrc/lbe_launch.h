@@ -145,23 +145,38 @@ cudaError_t launch_ghosts(const InstDev* d, int n_inst, int max_ny, int parity, 
 cudaError_t launch_seed_tick(uint32_t* seed, cudaStream_t s);
 cudaError_t launch_seed_set(uint32_t* seed, uint32_t value, cudaStream_t s);
 
-// Adjoint kernels (lbe_adjoint.cu), FP64, one instance d_one of nx x ny.
-// Scratch: adjoint_scratch_doubles(nx, ny) doubles.
-int64_t adjoint_scratch_doubles(int nx, int ny);
-// out4[0] = sum c u_y, out4[1] = sum c of the state Q[27][ny][nx] (device).
-cudaError_t launch_observable(const InstDev* d_one, int nx, int ny, const double* Q,
-                              double* scratch, double* out4, cudaStream_t s);
-// a_out = Post'(Q)^T Pull^T a_next + wl dl/dQ with obs = {sum c u_y, sum c} of
-// Q (device, read only if wl != 0); theta_acc[0..2] (device) += the parameter
-// partials.  a_next may be nullptr (zero).  fp32: the per-cell products in
-// FP32 arithmetic (the planes and the parameter sums stay FP64).
-cudaError_t launch_adjoint_step(const InstDev* d_one, int nx, int ny, const double* Q,
-                                const double* a_next, double wl, const double* obs,
-                                double* a_out, double* theta_acc, double* scratch, bool fp32,
-                                cudaStream_t s);
-// dT0[k] = rho c_v sum_i w_i a[18 + i][k]
-cudaError_t launch_adjoint_dT0(const InstDev* d_one, int nx, int ny, const double* a,
-                               double* dT0, cudaStream_t s);
+// Adjoint kernels (lbe_adjoint.cu), one instance d_one of nx x ny.  fp32:
+// states, adjoints and scratch are FP32 (a handle whose arithmetic is), else
+// FP64; sizes in planes of nx * ny values of adjoint_real_bytes.
+size_t adjoint_real_bytes(bool fp32);
+int64_t adjoint_state_planes(bool fp32);  // a state: populations and moments
+int64_t adjoint_vector_planes();          // an adjoint: 27 planes, then 3 terms of the cell
+int64_t adjoint_scratch_planes();
+int64_t adjoint_part_doubles(int nx, int ny);  // partial sums of the tiles
+// The state of buf[parity].
+cudaError_t launch_adjoint_state(int storage, const InstDev* d_one, int nx, int ny, int parity,
+                                 void* state, cudaStream_t s);
+// c, p, T (cpt[3][N]) of a caller's 27 FP64 planes.
+cudaError_t launch_adjoint_moments(const InstDev* d_one, int nx, int ny, const double* Q,
+                                   double* cpt, cudaStream_t s);
+// out4[0..1] = sum c u_y, sum c of a state.  fp32: Q is a state; else Q the 27
+// planes and cpt their moments.
+cudaError_t launch_observable(const InstDev* d_one, int nx, int ny, bool fp32, const void* Q,
+                              const void* cpt, double* part, double* out4, cudaStream_t s);
+// One adjoint step at the state (Q, cpt as above): aout (27 planes) and tout
+// (3 planes) from a, at (the same of the next state; at may be NULL: zero, a
+// NULL: a zero adjoint); part gains the theta sums of its tiles.
+cudaError_t launch_adjoint_step(const InstDev* d_one, int nx, int ny, bool fp32, const void* Q,
+                                const void* cpt, const void* a, const void* at, double wl,
+                                const double* obs, void* aout, void* tout, void* scratch,
+                                double* part, cudaStream_t s);
+// out4[0..2] = the theta sums.
+cudaError_t launch_adjoint_sums(const double* part, int nx, int ny, double* out4, cudaStream_t s);
+// 27 FP64 planes, and dL/dT0, of an adjoint.
+cudaError_t launch_adjoint_finish(int nx, int ny, bool fp32, const void* a, const void* at,
+                                  double* out, cudaStream_t s);
+cudaError_t launch_adjoint_dT0(const InstDev* d_one, int nx, int ny, bool fp32, const void* a,
+                               const void* at, double* dT0, cudaStream_t s);
 
 // Sets the message lbe_last_error(NULL) returns on this thread (lbe_api.cu).
 void set_thread_error(const char* msg);
