@@ -52,7 +52,8 @@ struct lbe_handle {
   InstDev* d_pinst = nullptr;    // [n] shape-0 work list of the pcorr pass (vrho)
   int64_t p_tiles = 0;           // its tiles
   int p_grid = 0;                // its CTAs
-  int tile = 0;
+  int tile = 0;                  // kernel id
+  int shape = 0;                 // tile kernel: the shape it runs (FP64: one of its own)
   int grid_req = 0;              // 0 = auto, -1 = one CTA per tile, >0 = CTAs
   int grid = 0;
   int seg_req = 0;               // strip kernel: rows per work item (0 = auto)
@@ -266,6 +267,21 @@ void fill_desc(lbe_handle* h, int j, InstDev& D) {
   D.pcorr = H.pcorr;
   D.uvel = H.uvel;
   P.eta_n2 = p.eta_n * p.eta_n;
+  // divisors: the rounded reciprocal and how a quotient is formed from it
+  auto den = [](double b, double& y, double& k) {
+    y = 1.0 / b;
+    const bool mid = b > std::ldexp(1.0, -60) && b < std::ldexp(1.0, 60);
+    const int kind = b == 1.0         ? 0
+                     : b == 1.0 / 3.0 ? 4
+                     : !mid           ? 3
+                     : std::fabs(std::fma(-b, y, 1.0)) <= std::ldexp(1.0, -54) ? 1 : 2;
+    const uint64_t bits = (uint64_t)kind;
+    memcpy(&k, &bits, sizeof k);
+  };
+  den(P.rcs2, P.yrcs2, P.krcs2);
+  den(P.rho, P.yrho, P.krho);
+  den(P.rcvcs2, P.yrcvcs2, P.krcvcs2);
+  den(P.rho_cv, P.yrcv, P.krcv);
   // hbar reference: linear profile between the mean wall temperatures
   double tb = 0, tt = 0;
   for (int x = 0; x < H.nx; x++) {
@@ -407,7 +423,10 @@ lbe_status setup_tiles(lbe_handle* h) {
     h->graph_failed = false;
     return wait(h);
   }
-  const TileShape ts = TILE_SHAPES[h->tile];
+  int max_nx = 0;
+  for (auto& H : h->inst) max_nx = std::max(max_nx, H.nx);
+  h->shape = h->storage != LBE_F64 ? h->tile : (max_nx <= NARROW_NX ? NARROW_TILE : F64_TILE);
+  const TileShape ts = TILE_SHAPES[h->shape];
   int64_t begin = 0;
   for (int j = 0; j < h->n; j++) {
     InstDev& D = h->idev[j];
@@ -419,7 +438,7 @@ lbe_status setup_tiles(lbe_handle* h) {
   h->total_tiles = begin;
   CU(h, cudaMemcpyAsync(h->d_inst, h->idev.data(), sizeof(InstDev) * h->n,
                         cudaMemcpyHostToDevice, h->stream));
-  const int occ = step_occupancy(h->storage, h->tile);
+  const int occ = step_occupancy(h->storage, h->shape);
   if (occ <= 0) return fail(h, LBE_ECUDA, "step kernel for tile %d cannot be resident", h->tile);
   if (h->grid_req == -1)
     h->grid = (int)(h->total_tiles < 2147483647 ? h->total_tiles : 2147483647);
@@ -464,7 +483,7 @@ cudaError_t launch_one_step(lbe_handle* h, int parity) {
             ? pcorr_f64(h->d_pinst, h->n, h->p_tiles, parity, h->p_grid, h->stream)
             : pcorr_f32(h->d_pinst, h->n, h->p_tiles, parity, h->p_grid, h->stream);
   if (e == cudaSuccess)
-    e = launch_step(h->storage, h->tile, h->d_inst, h->n, h->total_tiles, parity, h->grid,
+    e = launch_step(h->storage, h->shape, h->d_inst, h->n, h->total_tiles, parity, h->grid,
                     h->d_seed, h->stream);
   if (e == cudaSuccess) e = launch_seed_tick(h->d_seed, h->stream);
   return e;

@@ -1,22 +1,93 @@
 // Per-cell arithmetic of the fused step, shared by the tile kernel and the
 // strip kernel: isotropic stencils, chemical potential, CSF + Marangoni force,
 // velocity and the three forced BGK collisions (steps S2-S9).  Expressions are
-// evaluated in the operation order of the FP64 CPU reference; divisions are
-// true divisions in FP64 and products with a reciprocal in FP32 (dv()).
+// evaluated in the operation order of the FP64 CPU reference; divisions round
+// correctly in FP64 and are products with a reciprocal in FP32 (dv()).
 #pragma once
 
 #include "lbe_common.cuh"
 
 namespace lbe {
 
-// a / b: a true division in FP64 (parity mode rounds like the FP64
-// reference); a product with the precomputed reciprocal in FP32.
-__device__ __forceinline__ double dv(double a, double b, double) { return a / b; }
-__device__ __forceinline__ float dv(float a, float, float inv_b) { return a * inv_b; }
-
+// a / b in FP64, correctly rounded (parity mode rounds like the FP64
+// reference), for a divisor b > 0 whose rounded reciprocal y = RN(1/b) is at
+// hand: Markstein's iteration (P. Markstein, IBM J. Res. Dev. 34, 1990).  If q
+// is within one unit in the last place of a/b, the remainder r = a - b q is
+// exact and RN(q + r y) = RN(a/b).  q = RN(a y) is that close where the
+// residual |1 - b y| <= 2^-54 (kind 1: 3 operations); any other y needs one
+// more iteration first (kind 2: 5).  The true division takes about 10, and a
+// cell has 55 of them on a pipe with 1/64 of the FP32 rate.  Outside
+// 2^-900 <= |a| < 2^900, where a remainder could underflow, the true division.
+static __device__ __noinline__ double div_full(double a, double b) { return a / b; }
+template <int KIND>
+__device__ __forceinline__ double div_by(double a, double b, double y) {
+  const double q0 = a * y;
+  double q = fma(fma(-b, q0, a), y, q0);
+  if (KIND == 2) q = fma(fma(-b, q, a), y, q);
+  const unsigned hi = (unsigned)__double2hiint(a);
+  if (((hi >> 20) & 0x7ffu) - 123u < 1800u) return q;
+  // zero of the right sign (q is +0 for both)
+  if (((hi << 1) | (unsigned)__double2loint(a)) == 0u) return q0;
+  return div_full(a, b);
+}
+// a / fl(1/3), correctly rounded, in 2 operations.  fl(1/3) = (1 - 2^-54)/3, so
+// the quotient is 3 a + 3 a 2^-54 (1 + 2^-54 + ...), and 3 a is a multiple of a
+// quarter of the result's last place (ulp) while the second term lies between
+// a quarter and a half of it: rounding that term to a product and adding it in
+// one fused operation could miss a rounding boundary only where it is within
+// 2^-53 of ulp/4 or ulp/2, that is for 3 a next to a power of two, where
+// divisibility by 3 excludes the cases.  (Checked against the division for
+// every mantissa within 2^30 of those places.)
+__device__ __forceinline__ double dv_cs2(double a) {
+  const double q = fma(3.0, a, a * 0x1.8p-53);
+  const unsigned hi = (unsigned)__double2hiint(a);
+  // (for a zero q is the zero of the same sign)
+  if (((hi >> 20) & 0x7ffu) < 123u && ((hi << 1) | (unsigned)__double2loint(a)) != 0u)
+    return div_full(a, 1.0 / 3.0);
+  return q;
+}
+__device__ __forceinline__ float dv_cs2(float a) { return a * 3.f; }
 // c_s^2 = 1/3 of D2Q9
 template <class C>
 __device__ __forceinline__ C cs2() { return C(1.0 / 3.0); }
+
+// A divisor b: y = 1/b (FP64: rounded) and the kind: 1, 2 as above, 0 for b =
+// 1, 4 for b = fl(1/3), 3 for the true division.
+template <class C>
+struct Den {
+  C b, y;
+  int kind;
+};
+__device__ __forceinline__ double dv(double a, const Den<double>& d) {
+  if (d.kind == 0) return a;
+  if (d.kind == 4) return dv_cs2(a);
+  return d.kind == 1 ? div_by<1>(a, d.b, d.y) : (d.kind == 2 ? div_by<2>(a, d.b, d.y) : a / d.b);
+}
+__device__ __forceinline__ float dv(float a, const Den<float>& d) { return a * d.y; }
+__device__ __forceinline__ float dv(float a, float, float inv_b) { return a * inv_b; }
+// (the kind is stored in the low word of a constant)
+__device__ __forceinline__ Den<double> make_den(double b, double y, double k) {
+  return Den<double>{b, y, __double2loint(k)};
+}
+// The divisors of a cell: rho c_s^2, rho and rho c_v c_s^2 (rc: the density
+// of the cell, vr: it varies; then their reciprocals are formed here).
+template <class C>
+struct Dens {
+  Den<C> rcs2, rho, rcvcs2;
+};
+__device__ __forceinline__ Dens<double> make_dens(const Phys<double>& P, double rc, bool vr) {
+  if (vr) {
+    const double b = rc * (1.0 / 3.0), v = (rc * P.cv) * (1.0 / 3.0);
+    return Dens<double>{{b, 1.0 / b, 2}, {rc, 1.0 / rc, 2}, {v, 0.0, 3}};
+  }
+  return Dens<double>{make_den(P.rcs2, P.yrcs2, P.krcs2), make_den(P.rho, P.yrho, P.krho),
+                      make_den(P.rcvcs2, P.yrcvcs2, P.krcvcs2)};
+}
+__device__ __forceinline__ Dens<float> make_dens(const Phys<float>& P, float, bool) {
+  return Dens<float>{{P.rcs2, 3.f * P.inv_rho, 0},
+                     {P.rho, P.inv_rho, 0},
+                     {P.rcvcs2, 3.f * P.inv_rho_cv, 0}};
+}
 
 // Sum over i = 0..8: in index order in FP64 (the order of the FP64
 // reference), as a pairwise tree in FP32 (shorter dependency chains).
@@ -76,8 +147,8 @@ __device__ __forceinline__ void grad3(const C* rs, const C* rc, const C* rn, int
     // inheriting the rounding of the O(1) products w_i phi(x + xi_i)
     const C dEW = vE - vW, dNS = vN - vS;
     const C d1 = vNE - vSW, d2 = vSE - vNW;  // xi = (1, 1) and (1, -1)
-    gx = dv(wa * dEW + wd * (d1 + d2), cs2<C>(), C(3));
-    gy = dv(wa * dNS + wd * (d1 - d2), cs2<C>(), C(3));
+    gx = dv_cs2(wa * dEW + wd * (d1 + d2));
+    gy = dv_cs2(wa * dNS + wd * (d1 - d2));
   } else {
     C sx = wa * vE;
     sx = sx - wa * vW;
@@ -91,8 +162,8 @@ __device__ __forceinline__ void grad3(const C* rs, const C* rc, const C* rn, int
     sy = sy + wd * vNW;
     sy = sy - wd * vSW;
     sy = sy - wd * vSE;
-    gx = dv(sx, cs2<C>(), C(3));
-    gy = dv(sy, cs2<C>(), C(3));
+    gx = dv_cs2(sx);
+    gy = dv_cs2(sy);
   }
 }
 
@@ -108,14 +179,13 @@ __device__ __forceinline__ C lap3(const C* rs, const C* rc, const C* rn, int x) 
   t = t + wd * (rn[x - 1] - v0);
   t = t + wd * (rs[x - 1] - v0);
   t = t + wd * (rs[x + 1] - v0);
-  return dv(C(2) * t, cs2<C>(), C(3));
+  return dv_cs2(C(2) * t);
 }
 
 // Unit normal n = grad c / sqrt(|grad c|^2 + eta_n^2) (Eq. 3).
 template <class C>
 __device__ __forceinline__ void normal3(const C* rs, const C* rc, const C* rn, int x, C en2, C& nx,
-                                        C& ny) {
-  C gx, gy;
+                                        C& ny, C& gx, C& gy) {
   grad3(rs, rc, rn, x, gx, gy);
   const C inv = C(1) / sqrt(gx * gx + gy * gy + en2);
   nx = gx * inv;
@@ -135,8 +205,8 @@ __device__ __forceinline__ void grad3c(const float* rs, const float* rc, const f
   const float dNS = (rn[x] - rs[x]) + (lo_at(ln, x) - lo_at(ls, x));
   const float d1 = (rn[x + 1] - rs[x - 1]) + (lo_at(ln, x + 1) - lo_at(ls, x - 1));
   const float d2 = (rs[x + 1] - rn[x - 1]) + (lo_at(ls, x + 1) - lo_at(ln, x - 1));
-  gx = dv(wa * dEW + wd * (d1 + d2), cs2<float>(), 3.f);
-  gy = dv(wa * dNS + wd * (d1 - d2), cs2<float>(), 3.f);
+  gx = dv_cs2(wa * dEW + wd * (d1 + d2));
+  gy = dv_cs2(wa * dNS + wd * (d1 - d2));
 }
 __device__ __forceinline__ float lap3c(const float* rs, const float* rc, const float* rn,
                                        const __half* ls, const __half* lc, const __half* ln,
@@ -152,7 +222,7 @@ __device__ __forceinline__ float lap3c(const float* rs, const float* rc, const f
   t = t + wd * d(rn, ln, x - 1);
   t = t + wd * d(rs, ls, x - 1);
   t = t + wd * d(rs, ls, x + 1);
-  return dv(2.f * t, cs2<float>(), 3.f);
+  return dv_cs2(2.f * t);
 }
 __device__ __forceinline__ void normal3c(const float* rs, const float* rc, const float* rn,
                                          const __half* ls, const __half* lc, const __half* ln,
@@ -207,7 +277,7 @@ __device__ __forceinline__ Drive<S> drive(const Phys<typename S::C>& P, int gy,
   const C mar = -P.sigmaT * ea;
   // varying density (FP64 storage only): rho(c) in the body force, u, the
   // relaxation times, the equilibria and the sources
-  const bool vr = sizeof(C) == 8 && P.drho != C(0);
+  const bool vr = sizeof(C) == 8 && nonzero(P.drho);
   d.rho = vr ? rho_at(P, cc) : P.rho;
   d.dRx = vr ? (cs2<C>() * P.drho) * s.gcx : C(0);
   d.dRy = vr ? (cs2<C>() * P.drho) * s.gcy : C(0);
@@ -244,10 +314,9 @@ __device__ __forceinline__ Drive<S> drive(const Phys<typename S::C>& P, int gy,
     jy = jy - f[7];
     jy = jy - f[8];
   }
-  const C rho = d.rho, inv_rho = P.inv_rho;
-  const C rcs2 = vr ? d.rho * C(1.0 / 3.0) : P.rcs2, inv_rcs2 = C(3) * inv_rho;
-  d.ux = dv(jx, rcs2, inv_rcs2) + dv(C(0.5) * d.Fx, rho, inv_rho);
-  d.uy = dv(jy, rcs2, inv_rcs2) + dv(C(0.5) * d.Fy, rho, inv_rho);
+  const Dens<C> dn = make_dens(P, d.rho, vr);
+  d.ux = dv(jx, dn.rcs2) + dv(C(0.5) * d.Fx, dn.rho);
+  d.uy = dv(jy, dn.rcs2) + dv(C(0.5) * d.Fy, dn.rho);
   const C wa = WGT<C>(1), wd2 = C(2) * WGT<C>(5);
   if constexpr (sizeof(C) == 4) {
     // J = j + (w_axis + 2 w_diag) F as two floats (the force term, small
@@ -285,15 +354,15 @@ __device__ __forceinline__ void collide(const Phys<typename S::C>& P, const type
                                         typename S::C dhc = 0,
                                         const typename S::C* wdu = nullptr) {
   using C = typename S::C;
-  const bool vr = sizeof(C) == 8 && P.drho != C(0);  // varying density (FP64)
-  const C inv_rho = P.inv_rho;
-  const C rcs2 = vr ? d.rho * C(1.0 / 3.0) : P.rcs2, inv_rcs2 = C(3) * inv_rho;
+  const bool vr = sizeof(C) == 8 && nonzero(P.drho);  // varying density (FP64)
+  const Dens<C> dn = make_dens(P, d.rho, vr);
+  const C rcs2 = dn.rcs2.b, inv_rcs2 = dn.rcs2.y;
   // S3: properties, linear in c
   const C eta = prop_at(P, P.eta1, P.deta, P.eta2, P.ie1, P.ie2, cc);
   const C lam = prop_at(P, P.lam1, P.dlam, P.lam2, P.il1, P.il2, cc);
-  const C tau_f = dv(eta, rcs2, inv_rcs2) + C(0.5);
+  const C tau_f = dv(eta, dn.rcs2) + C(0.5);
   const C omega_f = C(1) / tau_f;
-  const C tau_h = dv(lam, vr ? (d.rho * P.cv) * C(1.0 / 3.0) : P.rcvcs2, C(3) * P.inv_rho_cv);
+  const C tau_h = dv(lam, dn.rcvcs2);
   const C omega_T = C(2) / (C(2) * tau_h + C(1));
   const C omega_g = P.omega_g;
   const C af = C(1) - C(0.5) * omega_f;
@@ -301,10 +370,10 @@ __device__ __forceinline__ void collide(const Phys<typename S::C>& P, const type
   const C aT = C(1) - C(0.5) * omega_T;
   const C ux = d.ux, uy = d.uy, Fx = d.Fx, Fy = d.Fy;
   // Gamma_i(u) = w_i (1 + xi.u/c_s^2 + ((xi.u/c_s^2)^2 - u^2/c_s^2)/2) (Eq. 6)
-  const C uu = dv(ux * ux + uy * uy, cs2<C>(), C(3));
+  const C uu = dv_cs2(ux * ux + uy * uy);
   const C Gm = P.Gm;
   // H_i of Eq. 22 (H_0 below, in the FP64 branch)
-  const C Hi = dv(Gm * d.mu, cs2<C>(), C(3));
+  const C Hi = dv_cs2(Gm * d.mu);
   const C Gx = Fx - gpx, Gy = Fy - gpy;  // F - grad p (= Fbar, uniform rho)
   const C rcvT = (vr ? d.rho : P.rho) * P.cv * (TT + d.Trow);  // rho c_v T (full T)
   const C rcvTr = P.rho_cv * d.Trow;            // rho c_v T_r(y)
@@ -494,8 +563,22 @@ __device__ __forceinline__ void collide(const Phys<typename S::C>& P, const type
       if (g0lo_out) *g0lo_out = lo_new;
     }
   } else {
-    const C H0 = dv(cc - dv((C(1) - WGT<C>(0)) * Gm * d.mu, cs2<C>(), C(3)), WGT<C>(0),
-                    C(9) / C(4));
+    const C H0 = dv(cc - dv_cs2((C(1) - WGT<C>(0)) * Gm * d.mu),
+                    Den<C>{WGT<C>(0), C(2.25), 1});  // (1/fl(4/9): residual 2^-54)
+    // xi_i.u/c_s^2: products by 0 and +-1 left out and opposite directions
+    // negated, which gives the sums of the FP64 reference but for the sign of
+    // a zero, which no use below sees (1 + xu, xu^2, and xu + hq, where hq is
+    // +0 if u is zero)
+    C xus[9];
+    xus[0] = C(0);
+    xus[1] = dv_cs2(ux);
+    xus[2] = dv_cs2(uy);
+    xus[5] = dv_cs2(ux + uy);
+    xus[6] = dv_cs2(uy - ux);
+    xus[3] = -xus[1];
+    xus[4] = -xus[2];
+    xus[7] = -xus[5];
+    xus[8] = -xus[6];
     // the pressure-work / viscous-dissipation term of Eq. aEq7 (wdu: the
     // cell's velocity gradients d_x u_x, d_y u_x, d_x u_y, d_y u_y), per
     // direction -fbar_i (xi_i - u).(xi_i.grad) u with fbar_i the density
@@ -508,10 +591,10 @@ __device__ __forceinline__ void collide(const Phys<typename S::C>& P, const type
 #pragma unroll
       for (int i = 0; i < 9; i++) {
         const C W = WGT<C>(i);
-        const C xu = dv(C(EX(i)) * ux + C(EY(i)) * uy, cs2<C>(), C(3));
+        const C xu = xus[i];
         const C G = W * (C(1) + xu + C(0.5) * (xu * xu - uu));
         const C fbe = d.rho * G;
-        const C fb = (f[i] - W * (pp - rcs2)) / cs2<C>();
+        const C fb = dv_cs2(f[i] - W * (pp - rcs2));
         const C fph = fbe + (C(1) - C(0.5) * omega_f) * (fb - fbe);
         const C dx = C(EX(i)) - ux, dy = C(EY(i)) - uy;
         const C q = dx * (C(EX(i)) * wdu[0] + C(EY(i)) * wdu[1]) +
@@ -523,7 +606,7 @@ __device__ __forceinline__ void collide(const Phys<typename S::C>& P, const type
 #pragma unroll
     for (int i = 0; i < 9; i++) {
       const C W = WGT<C>(i);
-      const C xu = dv(C(EX(i)) * ux + C(EY(i)) * uy, cs2<C>(), C(3));
+      const C xu = xus[i];
       const C hq = C(0.5) * (xu * xu - uu);
       const C G = W * (C(1) + xu + hq);
       const C q = xu + hq;  // velocity part, without the cancelling w_i
@@ -536,14 +619,14 @@ __device__ __forceinline__ void collide(const Phys<typename S::C>& P, const type
       out(0, i, f[i] - omega_f * (f[i] - feq) + af * fs);
       // g (Eq. 27 with Eq. 21-22)
       const C geq = W * ((i == 0 ? H0 : Hi) + cc * q);
-      const C gs = dv(cc * (dx * Gx + dy * Gy), rcs2, inv_rcs2) * G;
+      const C gs = dv(cc * (dx * Gx + dy * Gy), dn.rcs2) * G;
       out(1, i, g[i] - omega_g * (g[i] - geq) + ag * gs);
       // hbar (Eq. aEq12 with Eq. aEq9); deviation form:
       // h_eq - w_i rho c_v T_r = rho c_v (T' Gamma_i + T_r w_i q_i)
       const C heq = rcvT * G;
       // Fbar = grad(rho c_s^2) - grad p + F
       const C Hx = vr ? d.dRx + Gx : Gx, Hy = vr ? d.dRy + Gy : Gy;
-      const C hs = dv(Hx * dx + Hy * dy, rcs2, inv_rcs2) * heq;
+      const C hs = dv(Hx * dx + Hy * dy, dn.rcs2) * heq;
       const C heqd = dev_h<S>() ? rcvTd * G + rcvTr * (W * q) : heq;
       if (wdu)
         out(2, i, h[i] - omega_T * (h[i] - heqd) + aT * (hs + (ws[i] - W * ws0)) + W * ws0);

@@ -85,14 +85,24 @@ struct Phys {
   C harm, eta2, lam2, ie1, ie2, il1, il2;
   C wmid;
   C kw;
+  // FP64: 1/b rounded, and (in the low word) how a division by b is formed
+  // (lbe_cell.cuh: Den), for b = rho c_s^2, rho, rho c_v c_s^2, rho c_v
+  C yrcs2, krcs2, yrho, krho, yrcvcs2, krcvcs2, yrcv, krcv;
 };
+
+// v != 0 for a constant (no NaN): FP64 by its bits (a comparison would take a
+// slot of the FP64 pipe in every cell)
+__device__ __forceinline__ bool nonzero(float v) { return v != 0.f; }
+__device__ __forceinline__ bool nonzero(double v) {
+  return (((unsigned)__double2hiint(v) << 1) | (unsigned)__double2loint(v)) != 0u;
+}
 
 // eta(c) or lambda(c) between the phase values a (c = 0) and b (c = 1):
 // linear (a + c (b - a), d = b - a) or, with P.harm, harmonic
 // 1/((1 - c)/a + c/b) (ia, ib: the reciprocals, used by the FP32 forms).
 template <class C>
 __device__ __forceinline__ C prop_at(const Phys<C>& P, C a, C d, C b, C ia, C ib, C c) {
-  if (P.harm != C(0)) {
+  if (nonzero(P.harm)) {
     if constexpr (sizeof(C) == 8)
       return C(1) / ((C(1) - c) / a + c / b);
     else
@@ -106,13 +116,13 @@ __device__ __forceinline__ C prop_at(const Phys<C>& P, C a, C d, C b, C ia, C ib
 // c (1 - c) (Young's law through a cubic wall energy).
 template <class C>
 __device__ __forceinline__ C wet_ghost(const Phys<C>& P, C cm, int j) {
-  return P.kw != C(0) ? cm + C(2 * j + 1) * P.kw * cm * (C(1) - cm) : cm;
+  return nonzero(P.kw) ? cm + C(2 * j + 1) * P.kw * cm * (C(1) - cm) : cm;
 }
 
 // The density of a cell, linear in c: rho(c) = rho1 + c (rho2 - rho1).
 template <class C>
 __device__ __forceinline__ C rho_at(const Phys<C>& P, C c) {
-  return P.drho != C(0) ? P.rho + c * P.drho : P.rho;
+  return nonzero(P.drho) ? P.rho + c * P.drho : P.rho;
 }
 
 // Per-instance descriptor, built on the host, read by the kernels.

@@ -1036,7 +1036,9 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
         const C* cb = cring + o1;
         const C* cc2 = cring + o2;
         auto normal = [&](int j) {
-          normal3(ca, cb, cc2, j + 2, s_phys.eta_n2, nxr[nr(mn) + j + 2], nyr[nr(mn) + j + 2]);
+          C gx, gy;
+          normal3(ca, cb, cc2, j + 2, s_phys.eta_n2, nxr[nr(mn) + j + 2], nyr[nr(mn) + j + 2], gx,
+                  gy);
         };
         if (!helper) normal(t);
         // the halo columns x0 - 1 and x0 + NC

@@ -35,12 +35,15 @@ cudaError_t LBE_CAT(launch_step_, LBE_SUFFIX)(int tile, const InstDev* d, int n,
                                                int parity, int grid, const uint32_t* seed,
                                                cudaStream_t s) {
   switch (tile) {
-    case 0: return launch_one<32, 8>(d, n, total, parity, grid, seed, s);
 #if LBE_ALL_TILES
+    case 0: return launch_one<32, 8>(d, n, total, parity, grid, seed, s);
     case 1: return launch_one<64, 4>(d, n, total, parity, grid, seed, s);
     case 2: return launch_one<32, 16>(d, n, total, parity, grid, seed, s);
     case 3: return launch_one<64, 8>(d, n, total, parity, grid, seed, s);
     case 4: return launch_one<128, 4>(d, n, total, parity, grid, seed, s);
+#else
+    case NARROW_TILE: return launch_one<4, 8>(d, n, total, parity, grid, seed, s);
+    case F64_TILE: return launch_one<16, 8>(d, n, total, parity, grid, seed, s);
 #endif
     default: return cudaErrorInvalidValue;
   }
@@ -48,12 +51,15 @@ cudaError_t LBE_CAT(launch_step_, LBE_SUFFIX)(int tile, const InstDev* d, int n,
 
 int LBE_CAT(occupancy_, LBE_SUFFIX)(int tile) {
   switch (tile) {
-    case 0: return occ_one<32, 8>();
 #if LBE_ALL_TILES
+    case 0: return occ_one<32, 8>();
     case 1: return occ_one<64, 4>();
     case 2: return occ_one<32, 16>();
     case 3: return occ_one<64, 8>();
     case 4: return occ_one<128, 4>();
+#else
+    case NARROW_TILE: return occ_one<4, 8>();
+    case F64_TILE: return occ_one<16, 8>();
 #endif
     default: return 0;
   }

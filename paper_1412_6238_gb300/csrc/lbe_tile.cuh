@@ -17,6 +17,11 @@
 //       (lbe_cell.cuh).
 //   S10 store the 27 post-collision values at the cell (the pull of the next
 //       step streams them).
+// FP64 is bound by the FP64 pipe (2 lanes a cycle and SM; 77 % busy): 1,209 FP64
+// instructions per warp of cells with true divisions and comparisons of
+// constants, 790 with the quotients of lbe_cell.cuh, integer tests, opposite
+// directions sharing their parts and grad c taken from the normal pass (512 x
+// 1024: 1,282 -> 842 us a step with the tile shapes of lbe_launch.h).
 // At uniform density the grad(rho c_s^2) terms of Eq. 12, Eq. 13 and Fbar
 // vanish; with a density varying with c (FP64 storage) p is corrected by
 // (dt/2) u.grad(rho c_s^2) in a pass of its own (MODE 2), since the
@@ -71,12 +76,12 @@ __device__ __forceinline__ void pull9(const InstDev& I, const Phys<typename S::C
       // the wall temperature where the link crosses the wall (x - xi_x/2,
       // between the columns) when P.wmid, else at the cell's column
       C Twi = Tw;
-      if (P.wmid != C(0) && EX(i) != 0) {
+      if (nonzero(P.wmid) && EX(i) != 0) {
         int xs = q.x - EX(i);
         xs = xs < 0 ? xs + I.nx : (xs >= I.nx ? xs - I.nx : xs);
         Twi = C(0.5) * (Tw + wall_T<S>(I, xs, wb ? 0 : 1));
       }
-      return -v + C(2) * WGT<C>(i) * (P.drho != C(0) ? rho_cell : P.rho) * P.cv * Twi;
+      return -v + C(2) * WGT<C>(i) * (nonzero(P.drho) ? rho_cell : P.rho) * P.cv * Twi;
     }
     return v;
   };
@@ -140,6 +145,14 @@ __device__ __forceinline__ typename S::C ghost_T(const InstDev& I, int x, bool b
   return C(2) * wall_T<S>(I, x, bottom ? 2 : 3) - T;
 }
 
+// T = sum hbar / (rho c_v), rc the density of the cell
+__device__ __forceinline__ double cell_T(const Phys<double>& P, double h, double rc) {
+  return nonzero(P.drho) ? h / (rc * P.cv) : dv(h, make_den(P.rho_cv, P.yrcv, P.krcv));
+}
+__device__ __forceinline__ float cell_T(const Phys<float>& P, float h, float) {
+  return dv(h, P.rho_cv, P.inv_rho_cv);
+}
+
 // c, p, T at an arbitrary tile-region position: x wraps, rows beyond the
 // walls (gy in [-2, -1] or [ny, ny+1]) are ghosts.
 template <class S>
@@ -168,9 +181,9 @@ __device__ __forceinline__ void region_values(const InstDev& I, const Phys<typen
     const C rc = rho_at(P, cm);
     pull9<S, 0>(I, P, src, q, v);
     // p of Eq. 13: with a varying density, the corrected p of pcorr
-    p = (use_pcorr && P.drho != C(0)) ? (C)I.pcorr[(size_t)y * nx + q.x] : sum9(v);
+    p = (use_pcorr && nonzero(P.drho)) ? (C)I.pcorr[(size_t)y * nx + q.x] : sum9(v);
     pull9<S, 2, true>(I, P, src, q, v, rc);
-    T = P.drho != C(0) ? dv(sum9(v), rc * P.cv, C(1)) : dv(sum9(v), P.rho_cv, P.inv_rho_cv);
+    T = cell_T(P, sum9(v), rc);
     if (ghost != 0) T = ghost_T<S>(I, q.x, ghost < 0, T);
   } else {
     p = C(0);
@@ -196,6 +209,8 @@ struct Tile {
     C T[QH * QW];
     C nx[QH * QW];
     C ny[QH * QW];
+    // FP64: grad c of the cells, which the normals form anyway
+    C gx[sizeof(C) == 8 ? TX * TY : 1], gy[sizeof(C) == 8 ? TX * TY : 1];
   };
 
   __device__ static void run(const InstDev& I, int64_t tile, int parity, Smem& sm,
@@ -210,7 +225,7 @@ struct Tile {
     // the pre-pass has nothing to do for an instance without a varying
     // density (pcorr) or the dissipation term (uvel); the whole CTA leaves
     // together
-    const bool wants_p = P.drho != C(0) && I.pcorr != nullptr;
+    const bool wants_p = nonzero(P.drho) && I.pcorr != nullptr;
     if (MODE == 2 && !wants_p && I.uvel == nullptr) return;
 
     // ---- S1: own cell
@@ -232,8 +247,8 @@ struct Tile {
       const C rc = rho_at(P, cc);
       pull9<S, 2, true>(I, P, src, q, h, rc);
       // p of Eq. 13 (with a varying density the corrected p, MODE 2 / pcorr)
-      pp = (P.drho != C(0) && MODE == 0) ? (C)I.pcorr[(size_t)gy * nx + gx] : sum9(f);
-      TT = P.drho != C(0) ? dv(sum9(h), rc * P.cv, C(1)) : dv(sum9(h), P.rho_cv, P.inv_rho_cv);
+      pp = (nonzero(P.drho) && MODE == 0) ? (C)I.pcorr[(size_t)gy * nx + gx] : sum9(f);
+      TT = cell_T(P, sum9(h), rc);
     } else if (gy <= ny + 1) {
       region_values<S>(I, P, src, gx, gy, true, MODE == 0, cc, pp, TT);
     }
@@ -274,7 +289,12 @@ struct Tile {
     for (int r = tid; r < QW * QH; r += NT) {
       const int qx = r % QW, qy = r / QW;
       const C* c0 = sm.c + (qy + 1) * RW;
-      normal3(c0 - RW, c0, c0 + RW, qx + 1, en2, sm.nx[r], sm.ny[r]);
+      C gcx, gcy;
+      normal3(c0 - RW, c0, c0 + RW, qx + 1, en2, sm.nx[r], sm.ny[r], gcx, gcy);
+      if (sizeof(C) == 8 && qx > 0 && qx <= TX && qy > 0 && qy <= TY) {
+        sm.gx[(qy - 1) * TX + qx - 1] = gcx;
+        sm.gy[(qy - 1) * TX + qx - 1] = gcy;
+      }
     }
     __syncthreads();
 
@@ -282,7 +302,12 @@ struct Tile {
       Stencils<C> st;
       C d1, d2, dum;
       const C* c0 = sm.c + (ty + 2) * RW;
-      grad3(c0 - RW, c0, c0 + RW, tx + 2, st.gcx, st.gcy);
+      if constexpr (sizeof(C) == 8) {
+        st.gcx = sm.gx[tid];
+        st.gcy = sm.gy[tid];
+      } else {
+        grad3(c0 - RW, c0, c0 + RW, tx + 2, st.gcx, st.gcy);
+      }
       st.lapc = lap3(c0 - RW, c0, c0 + RW, tx + 2);
       const int qo = (ty + 1) * QW;
       grad3(sm.T + qo - QW, sm.T + qo, sm.T + qo + QW, tx + 1, st.gTx, st.gTy);
@@ -295,7 +320,7 @@ struct Tile {
       const Drive<S> d = drive<S>(P, gy, f, cc, TT, st);
 
       // Eq. 13 with a varying density: p = sum f_i + (dt/2) u.grad(rho c_s^2)
-      const C pcor = P.drho != C(0) ? pp + C(0.5) * (d.ux * d.dRx + d.uy * d.dRy) : pp;
+      const C pcor = nonzero(P.drho) ? pp + C(0.5) * (d.ux * d.dRx + d.uy * d.dRy) : pp;
       if (MODE == 2) {  // the corrected p and u for the step that follows
         const size_t k = (size_t)gy * nx + gx;
         if (wants_p) I.pcorr[k] = (double)pcor;
@@ -348,10 +373,10 @@ struct Tile {
           s2 += WGT<C>(i) * C(EX(i)) * vy;
           s3 += WGT<C>(i) * C(EY(i)) * vy;
         }
-        du[0] = dv(s0, cs2<C>(), C(3));
-        du[1] = dv(s1, cs2<C>(), C(3));
-        du[2] = dv(s2, cs2<C>(), C(3));
-        du[3] = dv(s3, cs2<C>(), C(3));
+        du[0] = dv_cs2(s0);
+        du[1] = dv_cs2(s1);
+        du[2] = dv_cs2(s2);
+        du[3] = dv_cs2(s3);
       }
       collide<S>(P, f, g, h, cc, pp, TT, st.gpx, st.gpy, d,
                  [&](int k, int i, C v) {
