@@ -17,7 +17,7 @@ bool tile_available(int storage, int tile) {
 }
 
 cudaError_t launch_stash(int storage, const InstDev* d, int n, int64_t items, int seg, int parity,
-                         int grid, int* err, int poll_lim, int withhold, const uint32_t* seed,
+                         int grid, int* err, int poll_lim, int withhold, StepCount seed,
                          bool var, bool own_ghosts, cudaStream_t s) {
   switch (storage) {
     case ST_F32:
@@ -47,7 +47,7 @@ int stash_occupancy(int storage) {
 }
 
 cudaError_t launch_step(int storage, int tile, const InstDev* d, int n, int64_t total, int parity,
-                        int grid, const uint32_t* seed, cudaStream_t s) {
+                        int grid, StepCount seed, cudaStream_t s) {
   switch (storage) {
     case ST_F64: return launch_step_f64(tile, d, n, total, parity, grid, seed, s);
     case ST_F32: return launch_step_f32(tile, d, n, total, parity, grid, seed, s);
@@ -308,9 +308,9 @@ constexpr int GHOST_PLANES = 20;
 // blockIdx.y: plane; blockIdx.x walks (instance, chunk of GHOST_THREADS / 2 XG
 // rows) pairs, chunks = row chunks of the tallest instance.
 __global__ void __launch_bounds__(GHOST_THREADS)
-ghost_kernel(const InstDev* __restrict__ insts, int n_inst, int chunks, int parity, uint32_t* seed) {
-  // the step is complete: advance the handle's step counter
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *seed += 1u;
+ghost_kernel(const InstDev* __restrict__ insts, int n_inst, int chunks, int parity) {
+  grid_wait();
+  grid_release();
   const int p = blockIdx.y;
   const int j = threadIdx.x % (2 * XG);
   const int64_t pairs = (int64_t)n_inst * chunks;
@@ -343,21 +343,20 @@ ghost_kernel(const InstDev* __restrict__ insts, int n_inst, int chunks, int pari
   }
 }
 
-cudaError_t launch_ghosts(const InstDev* d, int n_inst, int max_ny, int parity, uint32_t* seed,
-                          cudaStream_t s) {
+cudaError_t launch_ghosts(const InstDev* d, int n_inst, int max_ny, int parity, cudaStream_t s) {
   constexpr int rows = GHOST_THREADS / (2 * XG);
   const int chunks = (max_ny + rows - 1) / rows;
   const int64_t pairs = (int64_t)n_inst * chunks;
   const int bx = (int)std::min<int64_t>(pairs, 1 << 16);
-  ghost_kernel<<<dim3(bx, GHOST_PLANES), GHOST_THREADS, 0, s>>>(d, n_inst, chunks, parity, seed);
-  return cudaGetLastError();
+  return launch_early(ghost_kernel, dim3(bx, GHOST_PLANES), GHOST_THREADS, 0, s, d, n_inst, chunks,
+                      parity);
 }
 
 __global__ void seed_kernel(uint32_t* seed, uint32_t value, int set) {
-  *seed = set ? value : *seed + 1u;
+  *seed = set ? value : *seed + value;
 }
-cudaError_t launch_seed_tick(uint32_t* seed, cudaStream_t s) {
-  seed_kernel<<<1, 1, 0, s>>>(seed, 0u, 0);
+cudaError_t launch_seed_add(uint32_t* seed, uint32_t steps, cudaStream_t s) {
+  seed_kernel<<<1, 1, 0, s>>>(seed, steps, 0);
   return cudaGetLastError();
 }
 cudaError_t launch_seed_set(uint32_t* seed, uint32_t value, cudaStream_t s) {

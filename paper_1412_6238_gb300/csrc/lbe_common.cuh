@@ -125,6 +125,30 @@ __device__ __forceinline__ C rho_at(const Phys<C>& P, C c) {
   return nonzero(P.drho) ? P.rho + c * P.drho : P.rho;
 }
 
+// The number of a step: a handle's counter in device memory (the steps before
+// the current group of launches) and the step's place in the group, so that
+// the counter is advanced once per group and a captured group can be replayed.
+struct StepCount {
+  const uint32_t* base;
+  uint32_t ahead;
+#ifdef __CUDACC__
+  __device__ __forceinline__ uint32_t now() const { return __ldg(base) + ahead; }
+#endif
+};
+
+#ifdef __CUDACC__
+// Waits until the kernels before this one on the stream are complete and their
+// writes visible (no wait in a kernel that was launched the usual way).
+__device__ __forceinline__ void grid_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Lets the next kernel on the stream start (it waits in its own grid_wait).
+// Called after grid_wait, so that at most two kernels are under way.
+__device__ __forceinline__ void grid_release() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 // Per-instance descriptor, built on the host, read by the kernels.
 struct InstDev {
   int32_t nx, ny, pitch, tiles_x;

@@ -43,6 +43,30 @@ constexpr TileShape TILE_SHAPES[NUM_TILES + 2] = {{32, 8},  {64, 4},  {32, 16}, 
 inline bool is_strip(int tile) { return tile >= STRIP_FIRST && tile < NUM_TILES; }
 inline bool is_stash(int tile) { return tile == STASH_ID || tile == STASH_OWN_ID; }
 
+// Launches a kernel of a step so that it starts while the kernel before it on
+// the stream still runs: when that one calls grid_release in every CTA, or as
+// its last CTAs end.  It waits for its completion with grid_wait before it
+// touches device memory that a step writes or reads.  The launch, the start of
+// the CTAs and what comes before grid_wait are then off the critical path, on
+// which they are a good part of a small grid's step (us a step without / with
+// it: 96 x 64 FP32 8.6 / 7.1, 512 x 256 14.5 / 13.1, dissipation 512 x 256
+// 35.0 / 33.8, FP64 128 x 128 37.9 / 37.4; large grids equal).
+template <class... P, class... A>
+inline cudaError_t launch_early(void (*kernel)(P...), dim3 grid, int threads, size_t smem,
+                                cudaStream_t s, A... args) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Does the step kernel of this storage exist for this kernel id?
 bool tile_available(int storage, int tile);
 
@@ -53,28 +77,28 @@ bool tile_available(int storage, int tile);
 // are not issued, so that the waits for it run out.
 constexpr int STASH_POLLS = 1 << 22;       // polls of one bounded copy wait
 constexpr int STASH_POLLS_TEST = 1 << 12;  // with the withhold test hook
-// seed: the handle's step counter (device), read for the random bits of the
-// stochastic rounding of the 16-bit forms.  var: some instance uses a
+// seed: the step's number, read for the random bits of the stochastic
+// rounding of the 16-bit forms.  var: some instance uses a
 // boundary or property variant (the kernel built with them).
 cudaError_t launch_stash(int storage, const InstDev* d, int n, int64_t items, int seg, int parity,
-                         int grid, int* err, int poll_lim, int withhold, const uint32_t* seed,
+                         int grid, int* err, int poll_lim, int withhold, StepCount seed,
                          bool var, bool own_ghosts, cudaStream_t s);
 int stash_occupancy(int storage);
 cudaError_t launch_stash_f32(const InstDev* d, int n, int64_t items, int seg, int parity, int grid,
                              int* err, int poll_lim, int withhold,
-                             const uint32_t* seed, bool var,
+                             StepCount seed, bool var,
                              bool own_ghosts, cudaStream_t s);
 cudaError_t launch_stash_f16(const InstDev* d, int n, int64_t items, int seg, int parity, int grid,
                              int* err, int poll_lim, int withhold,
-                             const uint32_t* seed, bool var,
+                             StepCount seed, bool var,
                              bool own_ghosts, cudaStream_t s);
 cudaError_t launch_stash_bf16(const InstDev* d, int n, int64_t items, int seg, int parity,
                               int grid, int* err, int poll_lim, int withhold,
-                             const uint32_t* seed, bool var,
+                             StepCount seed, bool var,
                              bool own_ghosts, cudaStream_t s);
 cudaError_t launch_stash_mix(const InstDev* d, int n, int64_t items, int seg, int parity,
                              int grid, int* err, int poll_lim, int withhold,
-                             const uint32_t* seed, bool var,
+                             StepCount seed, bool var,
                              bool own_ghosts, cudaStream_t s);
 int stash_occupancy_f32();
 int stash_occupancy_f16();
@@ -84,7 +108,7 @@ int stash_occupancy_mix();
 // One step of every instance in d_inst[0..n_inst): persistent grid of `grid`
 // CTAs over total_tiles tiles; reads buf[parity], writes buf[parity ^ 1].
 cudaError_t launch_step(int storage, int tile, const InstDev* d_inst, int n_inst,
-                        int64_t total_tiles, int parity, int grid, const uint32_t* seed,
+                        int64_t total_tiles, int parity, int grid, StepCount seed,
                         cudaStream_t s);
 
 // Resident CTAs per SM of the step kernel (0 if unavailable).
@@ -97,15 +121,15 @@ cudaError_t launch_fields(int storage, const InstDev* d_one, int64_t tiles, int 
 
 // Per-storage entry points (defined in lbe_step_<storage>.cu).
 cudaError_t launch_step_f64(int tile, const InstDev* d, int n, int64_t total, int parity,
-                            int grid, const uint32_t* seed, cudaStream_t s);
+                            int grid, StepCount seed, cudaStream_t s);
 cudaError_t launch_step_f32(int tile, const InstDev* d, int n, int64_t total, int parity,
-                            int grid, const uint32_t* seed, cudaStream_t s);
+                            int grid, StepCount seed, cudaStream_t s);
 cudaError_t launch_step_f16(int tile, const InstDev* d, int n, int64_t total, int parity,
-                            int grid, const uint32_t* seed, cudaStream_t s);
+                            int grid, StepCount seed, cudaStream_t s);
 cudaError_t launch_step_bf16(int tile, const InstDev* d, int n, int64_t total, int parity,
-                             int grid, const uint32_t* seed, cudaStream_t s);
+                             int grid, StepCount seed, cudaStream_t s);
 cudaError_t launch_step_mix(int tile, const InstDev* d, int n, int64_t total, int parity,
-                            int grid, const uint32_t* seed, cudaStream_t s);
+                            int grid, StepCount seed, cudaStream_t s);
 int occupancy_f64(int tile);
 int occupancy_f32(int tile);
 int occupancy_f16(int tile);
@@ -146,12 +170,10 @@ cudaError_t launch_sums(const double* cur, const double* prev, int64_t n, double
 cudaError_t launch_f64_to_f32(const double* in, float* out, int64_t n, cudaStream_t s);
 // Periodic ghost columns of buffer `parity` of n_inst instances (16/32-bit
 // storages), after a step of the stash kernel.
-// (also advances the handle's step counter *seed by one)
-cudaError_t launch_ghosts(const InstDev* d, int n_inst, int max_ny, int parity, uint32_t* seed,
-                          cudaStream_t s);
-// The handle's step counter: +1 after every step (the ghost-column kernel
-// does it for the strip kernel; this one after a tile-kernel step), or set.
-cudaError_t launch_seed_tick(uint32_t* seed, cudaStream_t s);
+cudaError_t launch_ghosts(const InstDev* d, int n_inst, int max_ny, int parity, cudaStream_t s);
+// The handle's step counter (16-bit storages): advanced after the steps that
+// were launched with offsets to it, or set.
+cudaError_t launch_seed_add(uint32_t* seed, uint32_t steps, cudaStream_t s);
 cudaError_t launch_seed_set(uint32_t* seed, uint32_t value, cudaStream_t s);
 
 // Adjoint kernels (lbe_adjoint.cu), one instance d_one of nx x ny.  fp32:

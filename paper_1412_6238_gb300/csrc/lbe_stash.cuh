@@ -594,7 +594,7 @@ template <class S, int NC, bool VAR, bool OWN>
 __global__ void __launch_bounds__(StashCfg<S, NC, VAR>::THREADS, (StashCfg<S, NC, VAR>::MINB))
 stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items, int seg_rows,
              int parity, int* __restrict__ err, int poll_lim, int withhold,
-             const uint32_t* __restrict__ seed) {
+             const StepCount seed) {
   using Cfg = StashCfg<S, NC, VAR>;
   using Fmt = typename Cfg::Fmt;
   using C = float;
@@ -642,8 +642,6 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
   unsigned phase = 0;    // bit s: parity of the next completion of slot s
   unsigned ephase = 0;   // bit s: parity of the next release of slot s
   unsigned pending = 0;  // bit s: slot s has copies not yet waited for
-  // the handle's step counter (random bits of the stochastic rounding)
-  const uint32_t step = S::SR ? __ldg(seed) : 0u;
 
   // Work assignment.  seg_rows > 0: items of seg_rows rows of one strip
   // (tile_begin counts items), taken round-robin.  seg_rows <= 0: the rows
@@ -713,7 +711,6 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
       }
       return P;
     };
-    const uint32_t skey = S::SR ? sr_step_key(step, I.salt) : 0u;
     const size_t pitch = (size_t)I.pitch;
     const int x = x0 + own;
     const int xw = wrapx(x, nx);
@@ -788,6 +785,13 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
       }
       return ok;
     };
+
+    // the step before is complete from here on (its launch let this one start
+    // early: the barriers, the constants and the item are ready by now)
+    grid_wait();
+    grid_release();
+    // the step number (random bits of the stochastic rounding)
+    const uint32_t skey = S::SR ? sr_step_key(seed.now(), I.salt) : 0u;
 
     issue(ya - 2, false);
     // ring offsets of rows i - 2 .. i + 2, rotated from row to row

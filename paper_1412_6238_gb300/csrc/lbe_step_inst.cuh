@@ -15,11 +15,11 @@ namespace lbe {
 namespace {
 template <int TX, int TY>
 cudaError_t launch_one(const InstDev* d, int n, int64_t total, int parity, int grid,
-                       const uint32_t* seed, cudaStream_t s) {
+                       StepCount seed, cudaStream_t s) {
   if (grid <= 0) grid = 1;
   if ((int64_t)grid > total) grid = (int)total;
-  tile_kernel<LBE_ST, TX, TY, 0><<<grid, TX * TY, 0, s>>>(d, n, total, parity, nullptr, seed);
-  return cudaGetLastError();
+  return launch_early(tile_kernel<LBE_ST, TX, TY, 0>, dim3(grid), TX * TY, 0, s, d, n, total,
+                      parity, nullptr, seed);
 }
 template <int TX, int TY>
 int occ_one() {
@@ -32,7 +32,7 @@ int occ_one() {
 }  // namespace
 
 cudaError_t LBE_CAT(launch_step_, LBE_SUFFIX)(int tile, const InstDev* d, int n, int64_t total,
-                                               int parity, int grid, const uint32_t* seed,
+                                               int parity, int grid, StepCount seed,
                                                cudaStream_t s) {
   switch (tile) {
 #if LBE_ALL_TILES
@@ -72,8 +72,8 @@ cudaError_t LBE_CAT(pcorr_, LBE_SUFFIX)(const InstDev* d, int n, int64_t total, 
                                          int grid, cudaStream_t s) {
   if (grid <= 0) grid = 1;
   if ((int64_t)grid > total) grid = (int)total;
-  tile_kernel<LBE_ST, 32, 8, 2><<<grid, 256, 0, s>>>(d, n, total, parity, nullptr, nullptr);
-  return cudaGetLastError();
+  return launch_early(tile_kernel<LBE_ST, 32, 8, 2>, dim3(grid), 256, 0, s, d, n, total, parity,
+                      nullptr, StepCount{});
 }
 #endif
 
@@ -81,7 +81,7 @@ cudaError_t LBE_CAT(fields_, LBE_SUFFIX)(const InstDev* d, int64_t tiles, int pa
                                           cudaStream_t s) {
   if (tiles <= 0) return cudaSuccess;
   const unsigned grid = (unsigned)(tiles < 2147483647 ? tiles : 2147483647);
-  tile_kernel<LBE_ST, 32, 8, 1><<<grid, 256, 0, s>>>(d, 1, tiles, parity, out, nullptr);
+  tile_kernel<LBE_ST, 32, 8, 1><<<grid, 256, 0, s>>>(d, 1, tiles, parity, out, StepCount{});
   return cudaGetLastError();
 }
 
@@ -103,15 +103,14 @@ bool stash_attr() {
 }
 template <int NC, bool VAR, bool OWN>
 cudaError_t stash_one(const InstDev* d, int n, int64_t items, int seg, int parity, int grid,
-                      int* err, int poll_lim, int withhold, const uint32_t* seed,
+                      int* err, int poll_lim, int withhold, StepCount seed,
                       cudaStream_t s) {
   if (!stash_attr<NC, VAR, OWN>()) return cudaErrorInvalidValue;
   if (grid <= 0) grid = 1;
   if ((int64_t)grid > items) grid = (int)items;
-  stash_kernel<LBE_ST, NC, VAR, OWN>
-      <<<grid, StashCfg<LBE_ST, NC, VAR>::THREADS, StashCfg<LBE_ST, NC, VAR>::SMEM, s>>>(
-          d, n, items, seg, parity, err, poll_lim, withhold, seed);
-  return cudaGetLastError();
+  return launch_early(stash_kernel<LBE_ST, NC, VAR, OWN>, dim3(grid),
+                      StashCfg<LBE_ST, NC, VAR>::THREADS, StashCfg<LBE_ST, NC, VAR>::SMEM, s, d, n,
+                      items, seg, parity, err, poll_lim, withhold, seed);
 }
 template <int NC, bool VAR, bool OWN>
 int stash_occ() {
@@ -127,7 +126,7 @@ int stash_occ() {
 
 cudaError_t LBE_CAT(launch_stash_, LBE_SUFFIX)(const InstDev* d, int n, int64_t items, int seg,
                                                 int parity, int grid, int* err, int poll_lim,
-                                                int withhold, const uint32_t* seed, bool var,
+                                                int withhold, StepCount seed, bool var,
                                                 bool own_ghosts, cudaStream_t s) {
 #define LBE_STASH_ONE(V, O) \
   stash_one<128, V, O>(d, n, items, seg, parity, grid, err, poll_lim, withhold, seed, s)

@@ -404,11 +404,15 @@ struct Tile {
 template <class S, int TX, int TY, int MODE>
 __global__ void __launch_bounds__(TX * TY, (S::kind == ST_F64 || TX * TY >= 512) ? 1 : 2)
 tile_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_tiles, int parity,
-            double* __restrict__ out, const uint32_t* __restrict__ seed) {
+            double* __restrict__ out, const StepCount seed) {
   using T = Tile<S, TX, TY, MODE>;
   __shared__ typename T::Smem sm;
-  // the step counter of the handle (random bits of the stochastic rounding)
-  const uint32_t step = (S::SR && MODE == 0) ? __ldg(seed) : 0u;
+  // (no grid_release: the next step's CTAs are let in as the last of these end;
+  // let in early, they crowded the SMs that were done first, FP64 500 x 333
+  // with a density ratio 466 us a step against 449)
+  grid_wait();
+  // the step number (random bits of the stochastic rounding)
+  const uint32_t step = (S::SR && MODE == 0) ? seed.now() : 0u;
   for (int64_t t = blockIdx.x; t < total_tiles; t += gridDim.x) {
     int lo = 0, hi = n_inst - 1;
     while (lo < hi) {
