@@ -1,7 +1,7 @@
 #include <algorithm>
 // Auxiliary kernels: initial state, state conversion (push / pull between the
-// pre-collision form and a storage buffer), FP64 reductions, dtype casts,
-// and the storage dispatch of the step / field launchers.
+// pre-collision form and a storage buffer), FP64 reductions and
+// the storage dispatch of the step / field launchers.
 #include "lbe_launch.h"
 #include "lbe_tile.cuh"
 
@@ -69,8 +69,8 @@ int step_occupancy(int storage, int tile) {
   return 0;
 }
 
-cudaError_t launch_fields(int storage, const InstDev* d, int64_t tiles, int parity, double* out,
-                          cudaStream_t s) {
+cudaError_t launch_fields(int storage, const InstDev* d, int64_t tiles, int parity,
+                          const FieldOut& out, cudaStream_t s) {
   switch (storage) {
     case ST_F64: return fields_f64(d, tiles, parity, out, s);
     case ST_F32: return fields_f32(d, tiles, parity, out, s);
@@ -417,19 +417,6 @@ cudaError_t launch_sums(const double* cur, const double* prev, int64_t n, double
                         double* out, cudaStream_t s) {
   sums_pass1<<<SUM_BLOCKS, SUM_THREADS, 0, s>>>(cur, prev, n, partial);
   sums_pass2<<<1, SUM_THREADS, 0, s>>>(partial, out);
-  return cudaGetLastError();
-}
-
-__global__ void f64_to_f32_kernel(const double* __restrict__ in, float* __restrict__ out,
-                                  int64_t n) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x)
-    out[k] = (float)in[k];
-}
-cudaError_t launch_f64_to_f32(const double* in, float* out, int64_t n, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  const int grid = (int)((n + 255) / 256 < 65535 ? (n + 255) / 256 : 65535);
-  f64_to_f32_kernel<<<grid, 256, 0, s>>>(in, out, n);
   return cudaGetLastError();
 }
 

@@ -125,6 +125,23 @@ __device__ __forceinline__ C rho_at(const Phys<C>& P, C c) {
   return nonzero(P.drho) ? P.rho + c * P.drho : P.rho;
 }
 
+// Where the fields c, p, ux, uy, T of an instance go ([ny][nx] each; nullptr:
+// not wanted), as doubles or, with f32, rounded to floats.
+struct FieldOut {
+  void* to[5];
+  int f32;
+#ifdef __CUDACC__
+  template <class V>
+  __device__ __forceinline__ void put(int k, size_t at, V v) const {
+    if (to[k] == nullptr) return;
+    if (f32)
+      static_cast<float*>(to[k])[at] = (float)v;
+    else
+      static_cast<double*>(to[k])[at] = (double)v;
+  }
+#endif
+};
+
 // The number of a step: a handle's counter in device memory (the steps before
 // the current group of launches) and the step's place in the group, so that
 // the counter is advanced once per group and a captured group can be replayed.

@@ -115,9 +115,9 @@ cudaError_t launch_step(int storage, int tile, const InstDev* d_inst, int n_inst
 int step_occupancy(int storage, int tile);
 
 // Fields c, p, ux, uy, T of one instance (d_one, tiles of shape 0, whose
-// tile_begin must be 0) into out[5][ny][nx] (double).
+// tile_begin must be 0) into out.
 cudaError_t launch_fields(int storage, const InstDev* d_one, int64_t tiles, int parity,
-                          double* out, cudaStream_t s);
+                          const FieldOut& out, cudaStream_t s);
 
 // Per-storage entry points (defined in lbe_step_<storage>.cu).
 cudaError_t launch_step_f64(int tile, const InstDev* d, int n, int64_t total, int parity,
@@ -135,7 +135,8 @@ int occupancy_f32(int tile);
 int occupancy_f16(int tile);
 int occupancy_bf16(int tile);
 int occupancy_mix(int tile);
-cudaError_t fields_f64(const InstDev* d, int64_t tiles, int parity, double* out, cudaStream_t s);
+cudaError_t fields_f64(const InstDev* d, int64_t tiles, int parity, const FieldOut& out,
+                       cudaStream_t s);
 // Varying density (FP64 storage only): the corrected p of Eq. 13 of every
 // cell into each instance's pcorr; d is a work list of tile shape 0.
 cudaError_t pcorr_f64(const InstDev* d, int n, int64_t total, int parity, int grid,
@@ -143,10 +144,14 @@ cudaError_t pcorr_f64(const InstDev* d, int n, int64_t total, int parity, int gr
 // FP32 storage: the pre-pass of the dissipation term (u of every cell)
 cudaError_t pcorr_f32(const InstDev* d, int n, int64_t total, int parity, int grid,
                       cudaStream_t s);
-cudaError_t fields_f32(const InstDev* d, int64_t tiles, int parity, double* out, cudaStream_t s);
-cudaError_t fields_f16(const InstDev* d, int64_t tiles, int parity, double* out, cudaStream_t s);
-cudaError_t fields_bf16(const InstDev* d, int64_t tiles, int parity, double* out, cudaStream_t s);
-cudaError_t fields_mix(const InstDev* d, int64_t tiles, int parity, double* out, cudaStream_t s);
+cudaError_t fields_f32(const InstDev* d, int64_t tiles, int parity, const FieldOut& out,
+                       cudaStream_t s);
+cudaError_t fields_f16(const InstDev* d, int64_t tiles, int parity, const FieldOut& out,
+                       cudaStream_t s);
+cudaError_t fields_bf16(const InstDev* d, int64_t tiles, int parity, const FieldOut& out,
+                       cudaStream_t s);
+cudaError_t fields_mix(const InstDev* d, int64_t tiles, int parity, const FieldOut& out,
+                       cudaStream_t s);
 
 // Auxiliary kernels (lbe_aux.cu).
 // The rest state of every cell from c0, T0 (device, [ny][nx]) into
@@ -167,7 +172,6 @@ cudaError_t launch_pull(int storage, const InstDev* d_one, int nx, int ny, doubl
 int sums_blocks();
 cudaError_t launch_sums(const double* cur, const double* prev, int64_t n, double* partial,
                         double* out, cudaStream_t s);
-cudaError_t launch_f64_to_f32(const double* in, float* out, int64_t n, cudaStream_t s);
 // Periodic ghost columns of buffer `parity` of n_inst instances (16/32-bit
 // storages), after a step of the stash kernel.
 cudaError_t launch_ghosts(const InstDev* d, int n_inst, int max_ny, int parity, cudaStream_t s);

@@ -19,7 +19,7 @@ cudaError_t launch_one(const InstDev* d, int n, int64_t total, int parity, int g
   if (grid <= 0) grid = 1;
   if ((int64_t)grid > total) grid = (int)total;
   return launch_early(tile_kernel<LBE_ST, TX, TY, 0>, dim3(grid), TX * TY, 0, s, d, n, total,
-                      parity, nullptr, seed);
+                      parity, FieldOut{}, seed);
 }
 template <int TX, int TY>
 int occ_one() {
@@ -73,11 +73,11 @@ cudaError_t LBE_CAT(pcorr_, LBE_SUFFIX)(const InstDev* d, int n, int64_t total, 
   if (grid <= 0) grid = 1;
   if ((int64_t)grid > total) grid = (int)total;
   return launch_early(tile_kernel<LBE_ST, 32, 8, 2>, dim3(grid), 256, 0, s, d, n, total, parity,
-                      nullptr, StepCount{});
+                      FieldOut{}, StepCount{});
 }
 #endif
 
-cudaError_t LBE_CAT(fields_, LBE_SUFFIX)(const InstDev* d, int64_t tiles, int parity, double* out,
+cudaError_t LBE_CAT(fields_, LBE_SUFFIX)(const InstDev* d, int64_t tiles, int parity, const FieldOut& out,
                                           cudaStream_t s) {
   if (tiles <= 0) return cudaSuccess;
   const unsigned grid = (unsigned)(tiles < 2147483647 ? tiles : 2147483647);

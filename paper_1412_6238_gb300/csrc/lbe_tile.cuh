@@ -192,7 +192,7 @@ __device__ __forceinline__ void region_values(const InstDev& I, const Phys<typen
 }
 
 // Tile work.  MODE 0: full step (collide and store into the other buffer).
-// MODE 1: export c, p, ux, uy, T of the current state into out[5][ny][nx].
+// MODE 1: export the wanted ones of c, p, ux, uy, T of the current state.
 // MODE 2 (varying density): the corrected p of Eq. 13 of every cell into
 // I.pcorr, which MODE 0 then reads for p and its gradient.
 template <class S, int TX, int TY, int MODE>
@@ -214,7 +214,7 @@ struct Tile {
   };
 
   __device__ static void run(const InstDev& I, int64_t tile, int parity, Smem& sm,
-                             double* __restrict__ out, uint32_t step) {
+                             const FieldOut& out, uint32_t step) {
     const int tid = threadIdx.x;
     const int tx = tid % TX, ty = tid / TX;
     const int nx = I.nx, ny = I.ny;
@@ -331,12 +331,20 @@ struct Tile {
         return;
       }
       if (MODE == 1) {
-        const size_t N = (size_t)nx * ny, k = (size_t)gy * nx + gx;
-        out[k] = (double)cc + (double)clo;
-        out[N + k] = (double)pcor;
-        out[2 * N + k] = (double)d.ux;
-        out[3 * N + k] = (double)d.uy;
-        out[4 * N + k] = dev_h<S>() ? (double)TT + (I.hr0 + I.hr1 * gy) : (double)TT;
+        // bound by the populations' load and, where it has to convert, by the
+        // FP64 pipe (64 clocks a warp instruction): floats go out as floats
+        const size_t k = (size_t)gy * nx + gx;
+        if (S::kind != ST_F64 && out.f32)  // one rounding of the same sum:
+          out.put(0, k, cc + clo);         // in FP64 it is exact where it can matter
+        else
+          out.put(0, k, (double)cc + (double)clo);
+        out.put(1, k, pcor);
+        out.put(2, k, d.ux);
+        out.put(3, k, d.uy);
+        if constexpr (dev_h<S>())
+          out.put(4, k, (double)TT + (I.hr0 + I.hr1 * gy));
+        else
+          out.put(4, k, TT);
         return;
       }
 
@@ -404,7 +412,7 @@ struct Tile {
 template <class S, int TX, int TY, int MODE>
 __global__ void __launch_bounds__(TX * TY, (S::kind == ST_F64 || TX * TY >= 512) ? 1 : 2)
 tile_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_tiles, int parity,
-            double* __restrict__ out, const StepCount seed) {
+            const FieldOut out, const StepCount seed) {
   using T = Tile<S, TX, TY, MODE>;
   __shared__ typename T::Smem sm;
   // (no grid_release: the next step's CTAs are let in as the last of these end;

@@ -1,0 +1,52 @@
+"""Where and how fields may go: device buffers the kernel writes itself, in
+both types, all or some of them; and the ones that are copied to, at an address
+no double can be stored at, overlapping (written in order: the last one stays)
+and on the host.  All hold the same values: FP32 is the FP64 value rounded."""
+import ctypes
+
+import pytest
+import torch
+
+from paper_1412_6238_gb300 import workloads as wl
+from paper_1412_6238_gb300.lbe import FIELD_NAMES, LBE
+
+pytestmark = pytest.mark.gpu
+
+
+def export(sim, ptrs, on_device, dtype):
+    a = (ctypes.c_void_p * 5)(*ptrs)
+    mask = sum(1 << k for k in range(5) if ptrs[k])
+    sim._check(sim._L.lbe_fields(sim._h, 0, mask, a, on_device, dtype))
+
+
+@pytest.mark.parametrize("storage,nx,ny", [("f64", 33, 18), ("f32", 131, 20), ("f16mix", 4, 9),
+                                           ("f16dev", 32, 8), ("bf16dev", 65, 33)])
+def test_outputs_hold_the_same_values(storage, nx, ny):
+    w = wl.droplet(nx, ny, 4.0, nx / 2.0, ny / 2.0, Re=0.2, Ma=10.0, Ca=0.05, eta_m=0.2,
+                   eta_r=0.5, lam_r=0.5)
+    sim = LBE(w, storage=storage)
+    sim.step(5)
+    N = nx * ny
+    ref = sim.fields(device="cpu")
+    full = torch.stack([ref[k].reshape(-1) for k in FIELD_NAMES])
+    for dtype, code, size in ((torch.float64, 0, 8), (torch.float32, 1, 4)):
+        want = full.to(dtype)
+        for device in ("cuda", "cpu"):
+            buf = torch.full((5, N), -7.0, dtype=dtype, device=device)
+            export(sim, [buf[k].data_ptr() for k in range(5)], device == "cuda", code)
+            assert torch.equal(buf.cpu(), want)
+            buf.fill_(-7.0)
+            export(sim, [0, buf[1].data_ptr(), 0, 0, buf[4].data_ptr()], device == "cuda", code)
+            assert torch.equal(buf[[1, 4]].cpu(), want[[1, 4]])
+            assert (buf[[0, 2, 3]] == -7.0).all()
+            # one buffer for all, and each one cell on from the one before
+            export(sim, [buf[0].data_ptr()] * 5, device == "cuda", code)
+            assert torch.equal(buf[0].cpu(), want[4])
+            flat = torch.zeros(N + 4, dtype=dtype, device=device)
+            export(sim, [flat.data_ptr() + size * k for k in range(5)], device == "cuda", code)
+            assert torch.equal(flat[:4].cpu(), want[:4, 0])
+            assert torch.equal(flat[4:].cpu(), want[4])
+    # doubles at an address that is a multiple of four only
+    raw = torch.zeros(2 * N + 1, dtype=torch.float32, device="cuda")
+    export(sim, [raw.data_ptr() + 4, 0, 0, 0, 0], True, 0)
+    assert torch.equal(raw[1:].cpu().view(torch.float64), full[0])
