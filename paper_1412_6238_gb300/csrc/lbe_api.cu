@@ -429,9 +429,19 @@ lbe_status setup_tiles(lbe_handle* h) {
     h->graph_failed = false;
     return wait(h);
   }
-  int max_nx = 0;
-  for (auto& H : h->inst) max_nx = std::max(max_nx, H.nx);
-  h->shape = h->storage != LBE_F64 ? h->tile : (max_nx <= NARROW_NX ? NARROW_TILE : F64_TILE);
+  h->shape = h->tile;
+  if (h->storage == LBE_F64) {
+    int max_nx = 0;
+    int64_t split = 0;
+    const TileShape sp = TILE_SHAPES[SPLIT_TILE];
+    for (auto& H : h->inst) {
+      max_nx = std::max(max_nx, H.nx);
+      split += (int64_t)((H.nx + sp.tx - 1) / sp.tx) * ((H.ny + sp.ty - 1) / sp.ty);
+    }
+    h->shape = split <= (int64_t)SPLIT_PER_SM * h->num_sms ? SPLIT_TILE
+               : max_nx <= NARROW_NX                        ? NARROW_TILE
+                                                            : F64_TILE;
+  }
   const TileShape ts = TILE_SHAPES[h->shape];
   int64_t begin = 0;
   for (int j = 0; j < h->n; j++) {

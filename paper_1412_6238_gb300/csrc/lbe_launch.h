@@ -28,18 +28,24 @@ constexpr int STASH_OWN_ID = 8;
 // elements of up to 8 bytes from a strip start x0 <= nx - 1, against a
 // pitch of at least nx + 8 elements (at most 127 x 8 bytes)
 constexpr size_t ARENA_TAIL = 2048;
-// The shapes kernel 0 takes with FP64 storage: 4 x 8 cells when every instance
-// is at most NARROW_NX columns wide (in a 32 x 8 tile of a 4-column channel
-// every warp holds 4 cells, and the FP64 pipe takes a warp's instruction at
-// the same pace whether 4 lanes hold a cell or 32; 4 x 101: 46 us a step
-// against 93), else 16 x 8, of which two run side by side on an SM, so that one
+// The shapes kernel 0 takes with FP64 storage.  The FP64 pipe takes a warp's
+// instruction at the same pace whether 4 lanes hold a cell or 32.
+// SPLIT_TILE: 4 x 8 cells, their work divided among four warps (lbe_split.cuh),
+// while every SM has at most SPLIT_PER_SM of them.  us a step, 4 x 101 (13
+// tiles) 18, one warp a tile 39; 40 x 40 (50 tiles) 18.5, as 16 x 8 40.8; 96 x
+// 96 (288) 27, 38; but 128 x 100 (416) 48, 37.5.
+// NARROW_TILE: 4 x 8 cells by one warp, when every instance is at most
+// NARROW_NX columns wide (4 x 4800 48.5, split 59, as 16 x 8 125; 16 x 1300 51,
+// 74, 62).
+// F64_TILE: else 16 x 8, of which two run side by side on an SM, so that one
 // keeps the pipe busy at the other's barriers (512 x 1024: 842 us a step, 32 x
 // 8 896, 8 x 8 867; 128 x 128: 40, 62, 43).
-constexpr int NARROW_TILE = NUM_TILES, F64_TILE = NUM_TILES + 1;
+constexpr int NARROW_TILE = NUM_TILES, F64_TILE = NUM_TILES + 1, SPLIT_TILE = NUM_TILES + 2;
 constexpr int NARROW_NX = 16;
-constexpr TileShape TILE_SHAPES[NUM_TILES + 2] = {{32, 8},  {64, 4},  {32, 16}, {64, 8},
+constexpr int SPLIT_PER_SM = 2;
+constexpr TileShape TILE_SHAPES[NUM_TILES + 3] = {{32, 8},  {64, 4},  {32, 16}, {64, 8},
                                                   {128, 4}, {124, 0}, {60, 0},  {128, 0},
-                                                  {128, 0}, {4, 8},   {16, 8}};
+                                                  {128, 0}, {4, 8},   {16, 8},  {4, 8}};
 inline bool is_strip(int tile) { return tile >= STRIP_FIRST && tile < NUM_TILES; }
 inline bool is_stash(int tile) { return tile == STASH_ID || tile == STASH_OWN_ID; }
 

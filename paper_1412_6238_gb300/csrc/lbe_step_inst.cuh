@@ -1,10 +1,15 @@
 // Instantiation of the step / field kernels for one storage type.  Included
 // by lbe_step_<storage>.cu with LBE_ST (policy), LBE_SUFFIX and LBE_ALL_TILES
 // defined.
+#include <algorithm>
+
 #include "lbe_launch.h"
 #include "lbe_tile.cuh"
 #if LBE_STASH
 #include "lbe_stash.cuh"
+#endif
+#if !LBE_ALL_TILES  // FP64
+#include "lbe_split.cuh"
 #endif
 
 #define LBE_CAT2(a, b) a##b
@@ -42,6 +47,9 @@ cudaError_t LBE_CAT(launch_step_, LBE_SUFFIX)(int tile, const InstDev* d, int n,
     case 3: return launch_one<64, 8>(d, n, total, parity, grid, seed, s);
     case 4: return launch_one<128, 4>(d, n, total, parity, grid, seed, s);
 #else
+    case SPLIT_TILE:
+      grid = (int)std::min<int64_t>(std::max(grid, 1), total);
+      return launch_early(split_kernel, dim3(grid), SPLIT_THREADS, 0, s, d, n, total, parity);
     case NARROW_TILE: return launch_one<4, 8>(d, n, total, parity, grid, seed, s);
     case F64_TILE: return launch_one<16, 8>(d, n, total, parity, grid, seed, s);
 #endif
@@ -58,6 +66,11 @@ int LBE_CAT(occupancy_, LBE_SUFFIX)(int tile) {
     case 3: return occ_one<64, 8>();
     case 4: return occ_one<128, 4>();
 #else
+    case SPLIT_TILE: {
+      int b = 0;
+      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, split_kernel, SPLIT_THREADS, 0) ==
+                     cudaSuccess ? b : 0;
+    }
     case NARROW_TILE: return occ_one<4, 8>();
     case F64_TILE: return occ_one<16, 8>();
 #endif

@@ -191,6 +191,38 @@ __device__ __forceinline__ void region_values(const InstDev& I, const Phys<typen
   }
 }
 
+// Velocity gradients d_x u_x, d_y u_x, d_x u_y, d_y u_y of a cell from the
+// pre-pass's u (isotropic stencil in index order; no slip: the ghost rows hold
+// minus the mirror cell's u).
+template <class C>
+__device__ __forceinline__ void grad_u(const InstDev& I, int gx, int gy, C du[4]) {
+  const int nx = I.nx, ny = I.ny;
+  const size_t N = (size_t)nx * ny;
+  C s0 = C(0), s1 = C(0), s2 = C(0), s3 = C(0);
+  for (int i = 1; i < 9; i++) {
+    int xx = gx + EX(i), yy = gy + EY(i);
+    xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
+    C sg = C(1);
+    if (yy < 0) {
+      yy = -1 - yy;
+      sg = C(-1);
+    } else if (yy >= ny) {
+      yy = 2 * ny - 1 - yy;
+      sg = C(-1);
+    }
+    const size_t kk = (size_t)yy * nx + xx;
+    const C vx = sg * (C)I.uvel[kk], vy = sg * (C)I.uvel[N + kk];
+    s0 += WGT<C>(i) * C(EX(i)) * vx;
+    s1 += WGT<C>(i) * C(EY(i)) * vx;
+    s2 += WGT<C>(i) * C(EX(i)) * vy;
+    s3 += WGT<C>(i) * C(EY(i)) * vy;
+  }
+  du[0] = dv_cs2(s0);
+  du[1] = dv_cs2(s1);
+  du[2] = dv_cs2(s2);
+  du[3] = dv_cs2(s3);
+}
+
 // Tile work.  MODE 0: full step (collide and store into the other buffer).
 // MODE 1: export the wanted ones of c, p, ux, uy, T of the current state.
 // MODE 2 (varying density): the corrected p of Eq. 13 of every cell into
@@ -356,36 +388,9 @@ struct Tile {
           S::SR ? sr_cell(sr_step_key(step, I.salt), (uint32_t)gy * (uint32_t)nx + (uint32_t)gx)
                 : 0u;
       C gs = C(0);  // 16-bit forms: the stored moving g_i
-      // the dissipation term: velocity gradients from the pre-pass's u
-      // (isotropic stencil in index order; no slip: the ghost rows hold
-      // minus the mirror cell's u)
+      // the dissipation term
       C du[4] = {C(0), C(0), C(0), C(0)};
-      if (I.uvel != nullptr) {
-        const size_t N = (size_t)nx * ny;
-        C s0 = C(0), s1 = C(0), s2 = C(0), s3 = C(0);
-        for (int i = 1; i < 9; i++) {
-          int xx = gx + EX(i), yy = gy + EY(i);
-          xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
-          C sg = C(1);
-          if (yy < 0) {
-            yy = -1 - yy;
-            sg = C(-1);
-          } else if (yy >= ny) {
-            yy = 2 * ny - 1 - yy;
-            sg = C(-1);
-          }
-          const size_t kk = (size_t)yy * nx + xx;
-          const C vx = sg * (C)I.uvel[kk], vy = sg * (C)I.uvel[N + kk];
-          s0 += WGT<C>(i) * C(EX(i)) * vx;
-          s1 += WGT<C>(i) * C(EY(i)) * vx;
-          s2 += WGT<C>(i) * C(EX(i)) * vy;
-          s3 += WGT<C>(i) * C(EY(i)) * vy;
-        }
-        du[0] = dv_cs2(s0);
-        du[1] = dv_cs2(s1);
-        du[2] = dv_cs2(s2);
-        du[3] = dv_cs2(s3);
-      }
+      if (I.uvel != nullptr) grad_u(I, gx, gy, du);
       collide<S>(P, f, g, h, cc, pp, TT, st.gpx, st.gpy, d,
                  [&](int k, int i, C v) {
                    if constexpr (S::SR) {
