@@ -354,6 +354,24 @@ void free_handle(lbe_handle* h) {
   delete h;
 }
 
+// Rows per item of the strips (nc columns) of n instances: of lo..hi, the one
+// that minimises waves x (rows + warm), with `slots` items at a time.
+int item_rows(const InstHost* inst, int n, int nc, int64_t slots, int lo, int hi, int warm) {
+  double best = 1e300;
+  int rows = hi;
+  for (int seg = lo; seg <= hi; seg++) {
+    int64_t items = 0;
+    for (int j = 0; j < n; j++)
+      items += (int64_t)((inst[j].nx + nc - 1) / nc) * ((inst[j].ny + seg - 1) / seg);
+    const double cost = (double)((items + slots - 1) / slots) * (seg + warm);
+    if (cost < best * (1 - 1e-9)) {
+      best = cost;
+      rows = seg;
+    }
+  }
+  return rows;
+}
+
 // (Re)build the step descriptors for the current tile shape and upload them.
 lbe_status setup_tiles(lbe_handle* h) {
   if (is_strip(h->tile)) {
@@ -391,20 +409,7 @@ lbe_status setup_tiles(lbe_handle* h) {
       const int seg_lo = stash ? 1 : std::min(8, max_ny);
       const int seg_hi = stash ? std::min(96, max_ny) : max_ny;
       const int warm = stash ? 6 : 4;
-      double best = 1e300;
-      int best_seg = seg_hi;
-      for (int seg = seg_lo; seg <= seg_hi; seg++) {
-        int64_t items = 0;
-        for (auto& H : h->inst)
-          items += (int64_t)((H.nx + nc - 1) / nc) * ((H.ny + seg - 1) / seg);
-        const double waves = (double)((items + slots - 1) / slots);
-        const double cost = waves * (seg + warm);
-        if (cost < best * (1 - 1e-9)) {
-          best = cost;
-          best_seg = seg;
-        }
-      }
-      h->seg = best_seg;
+      h->seg = item_rows(h->inst.data(), h->n, nc, slots, seg_lo, seg_hi, warm);
     }
     // tile_begin: the instance's first item (seg > 0) or first strip row
     // (seg == 0: the rows of all strips end to end, tiles_y the band height
@@ -589,6 +594,20 @@ lbe_status ensure_scratch(lbe_handle* h) {
 
 lbe_status compute_fields(lbe_handle* h, int j, int which_parity, const FieldOut& out) {
   const InstHost& H = h->inst[j];
+  if (h->storage != LBE_F64 && H.nx >= XG) {
+    // the strip kernel's marching rows: 4096 x 4096 FP32 0.49 ms, the tile
+    // kernel (which pulls a ring of 2/3 of a tile's cells besides) 1.79
+    const int nc = TILE_SHAPES[STASH_ID].tx;
+    const int occ = stash_occupancy(h->storage);
+    if (occ <= 0) return fail(h, LBE_ECUDA, "the field kernel cannot be resident");
+    const int grid = occ * h->num_sms;
+    const int seg = item_rows(&H, 1, nc, grid, 1, std::min(96, H.ny), 6);
+    const int64_t items = (int64_t)((H.nx + nc - 1) / nc) * ((H.ny + seg - 1) / seg);
+    cudaError_t e = launch_strip_fields(h->storage, h->d_finst + j, items, seg, which_parity, grid,
+                                        h->d_err, h->variants, out, h->stream);
+    if (e != cudaSuccess) return fail(h, LBE_ECUDA, "field kernel: %s", cudaGetErrorString(e));
+    return LBE_OK;
+  }
   const TileShape ts = TILE_SHAPES[0];
   const int64_t tiles = (int64_t)((H.nx + ts.tx - 1) / ts.tx) * ((H.ny + ts.ty - 1) / ts.ty);
   cudaError_t e = launch_fields(h->storage, h->d_finst + j, tiles, which_parity, out, h->stream);

@@ -36,6 +36,18 @@ cudaError_t launch_stash(int storage, const InstDev* d, int n, int64_t items, in
   return cudaErrorInvalidValue;
 }
 
+cudaError_t launch_strip_fields(int storage, const InstDev* d, int64_t items, int seg, int parity,
+                                int grid, int* err, bool var, const FieldOut& out,
+                                cudaStream_t s) {
+  switch (storage) {
+    case ST_F32: return strip_fields_f32(d, items, seg, parity, grid, err, var, out, s);
+    case ST_F16DEV: return strip_fields_f16(d, items, seg, parity, grid, err, var, out, s);
+    case ST_BF16DEV: return strip_fields_bf16(d, items, seg, parity, grid, err, var, out, s);
+    case ST_F16MIX: return strip_fields_mix(d, items, seg, parity, grid, err, var, out, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
 int stash_occupancy(int storage) {
   switch (storage) {
     case ST_F32: return stash_occupancy_f32();

@@ -89,6 +89,11 @@ constexpr int STASH_POLLS_TEST = 1 << 12;  // with the withhold test hook
 cudaError_t launch_stash(int storage, const InstDev* d, int n, int64_t items, int seg, int parity,
                          int grid, int* err, int poll_lim, int withhold, StepCount seed,
                          bool var, bool own_ghosts, cudaStream_t s);
+// The same kernel's fields of one instance (d_one, tile_begin 0) over `items`
+// work items of seg rows of a strip.
+cudaError_t launch_strip_fields(int storage, const InstDev* d_one, int64_t items, int seg,
+                                int parity, int grid, int* err, bool var, const FieldOut& out,
+                                cudaStream_t s);
 int stash_occupancy(int storage);
 cudaError_t launch_stash_f32(const InstDev* d, int n, int64_t items, int seg, int parity, int grid,
                              int* err, int poll_lim, int withhold,
@@ -106,6 +111,14 @@ cudaError_t launch_stash_mix(const InstDev* d, int n, int64_t items, int seg, in
                              int grid, int* err, int poll_lim, int withhold,
                              StepCount seed, bool var,
                              bool own_ghosts, cudaStream_t s);
+cudaError_t strip_fields_f32(const InstDev* d, int64_t items, int seg, int parity, int grid,
+                            int* err, bool var, const FieldOut& out, cudaStream_t s);
+cudaError_t strip_fields_f16(const InstDev* d, int64_t items, int seg, int parity, int grid,
+                            int* err, bool var, const FieldOut& out, cudaStream_t s);
+cudaError_t strip_fields_bf16(const InstDev* d, int64_t items, int seg, int parity, int grid,
+                            int* err, bool var, const FieldOut& out, cudaStream_t s);
+cudaError_t strip_fields_mix(const InstDev* d, int64_t items, int seg, int parity, int grid,
+                            int* err, bool var, const FieldOut& out, cudaStream_t s);
 int stash_occupancy_f32();
 int stash_occupancy_f16();
 int stash_occupancy_bf16();

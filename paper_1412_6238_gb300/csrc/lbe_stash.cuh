@@ -590,11 +590,13 @@ __device__ __forceinline__ void next_plane(char*& p, uint64_t plane) {
 // OWN: the kernel writes the periodic ghost columns of its output itself
 // (a compile-time choice: compiled in, the ghost stores cost the main
 // stores about 1 % even where no lane takes them).
-template <class S, int NC, bool VAR, bool OWN>
+// EXPORT: instead of colliding, the fields of the cells into `out` (the work
+// list is then one instance, the items of seg_rows rows of its strips).
+template <class S, int NC, bool VAR, bool OWN, bool EXPORT>
 __global__ void __launch_bounds__(StashCfg<S, NC, VAR>::THREADS, (StashCfg<S, NC, VAR>::MINB))
 stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items, int seg_rows,
              int parity, int* __restrict__ err, int poll_lim, int withhold,
-             const StepCount seed) {
+             const StepCount seed, const FieldOut out) {
   using Cfg = StashCfg<S, NC, VAR>;
   using Fmt = typename Cfg::Fmt;
   using C = float;
@@ -691,8 +693,9 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
       }
       g += yb - ya;
     } else {
-      strip = (int)(local % I.tiles_x);
-      ya = (int)(local / I.tiles_x) * seg_rows;
+      const int ns = EXPORT ? (nx + Cfg::NCO - 1) / Cfg::NCO : I.tiles_x;
+      strip = (int)(local % ns);
+      ya = (int)(local / ns) * seg_rows;
       yb = min(ya + seg_rows, ny);
       g += gridDim.x;
     }
@@ -855,83 +858,87 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
         grad3(nyr + ns, nyr + n0, nyr + nn, t, dum, d2);
         st.kappa = d1 + d2;
         const Drive<S> d = drive<S>(P, r, f, cc, TT, st);
-        C o[27];
-        C lo_out = C(0);
-        const C dhc = (r > 0 && r < I.ny - 1) ? P.dh : C(0);
-        collide<S>(P, f, g, h, cc, pp, TT, st.gpx, st.gpy, d,
-                   [&](int k, int ii, C v) { o[k * 9 + ii] = v; }, g0lo, clo, &lo_out, dhc);
-        // 16-bit forms: the cell's random bits for the stochastic rounding
-        const uint32_t hc = S::SR ? sr_cell(skey, (uint32_t)r * (uint32_t)nx + (uint32_t)x) : 0u;
-        // the cell's values stored at its element and, with OWN, by the lanes
-        // of the periodic edge columns at its ghost copies (the 16-bit forms
-        // round them again, with the same random bits: the same values)
-        auto store_at = [&](const size_t e) {
-          if constexpr (MIX) {
-            // word i: (f_i, g_i, hbar_i); word 0: (f_0, hbar_0, g_0 low part)
-            const float s1 = I.s[1], s2 = I.s[2];
-            float gs = 0.f;  // the stored g_i, times s_1
-            char* const w0 = dst + 8 * e;
-            char* w = w0;
+        if constexpr (EXPORT) {
+          put_fields<S>(out, I, (size_t)r * nx + x, r, cc, clo, pp, TT, d);
+        } else {
+          C o[27];
+          C lo_out = C(0);
+          const C dhc = (r > 0 && r < I.ny - 1) ? P.dh : C(0);
+          collide<S>(P, f, g, h, cc, pp, TT, st.gpx, st.gpy, d,
+                     [&](int k, int ii, C v) { o[k * 9 + ii] = v; }, g0lo, clo, &lo_out, dhc);
+          // 16-bit forms: the cell's random bits for the stochastic rounding
+          const uint32_t hc = S::SR ? sr_cell(skey, (uint32_t)r * (uint32_t)nx + (uint32_t)x) : 0u;
+          // the cell's values stored at its element and, with OWN, by the lanes
+          // of the periodic edge columns at its ghost copies (the 16-bit forms
+          // round them again, with the same random bits: the same values)
+          auto store_at = [&](const size_t e) {
+            if constexpr (MIX) {
+              // word i: (f_i, g_i, hbar_i); word 0: (f_0, hbar_0, g_0 low part)
+              const float s1 = I.s[1], s2 = I.s[2];
+              float gs = 0.f;  // the stored g_i, times s_1
+              char* const w0 = dst + 8 * e;
+              char* w = w0;
 #pragma unroll
-            for (int ii = 1; ii < 9; ii++) {
-              const uint32_t q =
-                  sr_pack_half2(o[9 + ii] * s1, o[18 + ii] * s2, S::sr_word(1, ii, hc));
-              gs += __half2float(__ushort_as_half((unsigned short)(q & 0xffffu)));
-              next_plane(w, I.pair_bytes);
-              *reinterpret_cast<uint2*>(w) = make_uint2(__float_as_uint(o[ii]), q);
-            }
-            float g0h, g0l;
-            g0_remainder(cc, clo, gs * P.inv_s[1], g0h, g0l);
-            *reinterpret_cast<uint2*>(w0) = make_uint2(
-                __float_as_uint(o[0]),
-                (uint32_t)__half_as_ushort(sr_half(o[18] * s2, S::sr_word(2, 0, hc))) |
-                    ((uint32_t)__half_as_ushort(__float2half_rn(g0l * G0LO_SCALE)) << 16));
-            reinterpret_cast<float*>(dst + I.g0_off)[e] = g0h;
-          } else if constexpr (!W16) {
-            st_g0lo<S>(I, dst, e, lo_out);
-            char* w = dst + 8 * e;
+              for (int ii = 1; ii < 9; ii++) {
+                const uint32_t q =
+                    sr_pack_half2(o[9 + ii] * s1, o[18 + ii] * s2, S::sr_word(1, ii, hc));
+                gs += __half2float(__ushort_as_half((unsigned short)(q & 0xffffu)));
+                next_plane(w, I.pair_bytes);
+                *reinterpret_cast<uint2*>(w) = make_uint2(__float_as_uint(o[ii]), q);
+              }
+              float g0h, g0l;
+              g0_remainder(cc, clo, gs * P.inv_s[1], g0h, g0l);
+              *reinterpret_cast<uint2*>(w0) = make_uint2(
+                  __float_as_uint(o[0]),
+                  (uint32_t)__half_as_ushort(sr_half(o[18] * s2, S::sr_word(2, 0, hc))) |
+                      ((uint32_t)__half_as_ushort(__float2half_rn(g0l * G0LO_SCALE)) << 16));
+              reinterpret_cast<float*>(dst + I.g0_off)[e] = g0h;
+            } else if constexpr (!W16) {
+              st_g0lo<S>(I, dst, e, lo_out);
+              char* w = dst + 8 * e;
 #pragma unroll
-            for (int ii = 0; ii < 9; ii++) {
-              *reinterpret_cast<float2*>(w) = make_float2(o[ii], o[9 + ii]);
-              next_plane(w, I.pair_bytes);
-            }
-            w = dst + I.h_off + 4 * e;
+              for (int ii = 0; ii < 9; ii++) {
+                *reinterpret_cast<float2*>(w) = make_float2(o[ii], o[9 + ii]);
+                next_plane(w, I.pair_bytes);
+              }
+              w = dst + I.h_off + 4 * e;
 #pragma unroll
-            for (int ii = 0; ii < 9; ii++) {
-              *reinterpret_cast<float*>(w) = o[18 + ii];
-              next_plane(w, I.plane_bytes);
-            }
-          } else {
-            S::st_sr(I, dst, 0, 0, e, o[0], S::sr_word(0, 0, hc));
-            float gs = 0.f;  // the stored g_i, times s_1
-            const float s0 = I.s[0], s1 = I.s[1], s2 = I.s[2];
-            char* w = dst + 4 * e;
+              for (int ii = 0; ii < 9; ii++) {
+                *reinterpret_cast<float*>(w) = o[18 + ii];
+                next_plane(w, I.plane_bytes);
+              }
+            } else {
+              S::st_sr(I, dst, 0, 0, e, o[0], S::sr_word(0, 0, hc));
+              float gs = 0.f;  // the stored g_i, times s_1
+              const float s0 = I.s[0], s1 = I.s[1], s2 = I.s[2];
+              char* w = dst + 4 * e;
 #pragma unroll
-            for (int ii = 1; ii < 9; ii++) {
-              const uint32_t q = S::sr_pack(o[ii] * s0, o[9 + ii] * s1, S::sr_word(0, ii, hc));
-              gs += S::pack_hi(q);
-              *reinterpret_cast<uint32_t*>(w) = q;
-              next_plane(w, I.pair_bytes);
-            }
-            float g0h, g0l;
-            g0_remainder(cc, clo, gs * P.inv_s[1], g0h, g0l);
-            S::st(I, dst, 1, 0, e, g0h);
-            st_g0lo<S>(I, dst, e, g0l);
-            w = dst + I.h_off + 2 * e;
+              for (int ii = 1; ii < 9; ii++) {
+                const uint32_t q = S::sr_pack(o[ii] * s0, o[9 + ii] * s1, S::sr_word(0, ii, hc));
+                gs += S::pack_hi(q);
+                *reinterpret_cast<uint32_t*>(w) = q;
+                next_plane(w, I.pair_bytes);
+              }
+              float g0h, g0l;
+              g0_remainder(cc, clo, gs * P.inv_s[1], g0h, g0l);
+              S::st(I, dst, 1, 0, e, g0h);
+              st_g0lo<S>(I, dst, e, g0l);
+              w = dst + I.h_off + 2 * e;
 #pragma unroll
-            for (int ii = 0; ii < 9; ii++) {
-              *reinterpret_cast<typename Fmt::E*>(w) =
-                  S::sr_one(o[18 + ii] * s2, S::sr_word(2, ii, hc));
-              next_plane(w, I.plane_bytes);
+              for (int ii = 0; ii < 9; ii++) {
+                *reinterpret_cast<typename Fmt::E*>(w) =
+                    S::sr_one(o[18 + ii] * s2, S::sr_word(2, ii, hc));
+                next_plane(w, I.plane_bytes);
+              }
             }
-          }
-        };
-        store_at((size_t)r * pitch + XG + x);
-        if constexpr (OWN) {
-          if (ndst > 1) {
+          };
+          store_at((size_t)r * pitch + XG + x);
+          if constexpr (OWN) {
+            if (ndst > 1) {
 #pragma unroll 1
-            for (int dq = 1; dq < ndst; dq++)
-              store_at((size_t)r * pitch + (XG + x + ((dq == 1 && gR) ? nx : -nx)));
+              for (int dq = 1; dq < ndst; dq++)
+                store_at((size_t)r * pitch + (XG + x + ((dq == 1 && gR) ? nx : -nx)));
+            }
           }
         }
       } else if (!helper) {

@@ -100,13 +100,13 @@ cudaError_t LBE_CAT(fields_, LBE_SUFFIX)(const InstDev* d, int64_t tiles, int pa
 
 #if LBE_STASH
 namespace {
-template <int NC, bool VAR, bool OWN>
+template <int NC, bool VAR, bool OWN, bool EXPORT = false>
 bool stash_attr() {
   static bool done[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
   if (!done[dev]) {
-    if (cudaFuncSetAttribute(stash_kernel<LBE_ST, NC, VAR, OWN>,
+    if (cudaFuncSetAttribute(stash_kernel<LBE_ST, NC, VAR, OWN, EXPORT>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                              StashCfg<LBE_ST, NC, VAR>::SMEM) != cudaSuccess)
       return false;
@@ -121,21 +121,39 @@ cudaError_t stash_one(const InstDev* d, int n, int64_t items, int seg, int parit
   if (!stash_attr<NC, VAR, OWN>()) return cudaErrorInvalidValue;
   if (grid <= 0) grid = 1;
   if ((int64_t)grid > items) grid = (int)items;
-  return launch_early(stash_kernel<LBE_ST, NC, VAR, OWN>, dim3(grid),
+  return launch_early(stash_kernel<LBE_ST, NC, VAR, OWN, false>, dim3(grid),
                       StashCfg<LBE_ST, NC, VAR>::THREADS, StashCfg<LBE_ST, NC, VAR>::SMEM, s, d, n,
-                      items, seg, parity, err, poll_lim, withhold, seed);
+                      items, seg, parity, err, poll_lim, withhold, seed, FieldOut{});
+}
+// the fields of one instance (d), seg rows an item
+template <bool VAR>
+cudaError_t stash_fields(const InstDev* d, int64_t items, int seg, int parity, int grid, int* err,
+                         const FieldOut& out, cudaStream_t s) {
+  using Cfg = StashCfg<LBE_ST, 128, VAR>;
+  if (!stash_attr<128, VAR, false, true>()) return cudaErrorInvalidValue;
+  stash_kernel<LBE_ST, 128, VAR, false, true>
+      <<<(int)std::min<int64_t>(grid, items), Cfg::THREADS, Cfg::SMEM, s>>>(
+          d, 1, items, seg, parity, err, STASH_POLLS, -1, StepCount{}, out);
+  return cudaGetLastError();
 }
 template <int NC, bool VAR, bool OWN>
 int stash_occ() {
   if (!stash_attr<NC, VAR, OWN>()) return 0;
   int b = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, stash_kernel<LBE_ST, NC, VAR, OWN>,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, stash_kernel<LBE_ST, NC, VAR, OWN, false>,
                                                     StashCfg<LBE_ST, NC, VAR>::THREADS,
                                                     StashCfg<LBE_ST, NC, VAR>::SMEM) != cudaSuccess)
     return 0;
   return b;
 }
 }  // namespace
+
+cudaError_t LBE_CAT(strip_fields_, LBE_SUFFIX)(const InstDev* d, int64_t items, int seg,
+                                                int parity, int grid, int* err, bool var,
+                                                const FieldOut& out, cudaStream_t s) {
+  return var ? stash_fields<true>(d, items, seg, parity, grid, err, out, s)
+             : stash_fields<false>(d, items, seg, parity, grid, err, out, s);
+}
 
 cudaError_t LBE_CAT(launch_stash_, LBE_SUFFIX)(const InstDev* d, int n, int64_t items, int seg,
                                                 int parity, int grid, int* err, int poll_lim,

@@ -191,6 +191,26 @@ __device__ __forceinline__ void region_values(const InstDev& I, const Phys<typen
   }
 }
 
+// The fields of the cell in row y, number k of the instance.  Where a value has
+// to be converted, the FP64 pipe takes 64 clocks a warp instruction: floats go
+// out as floats.
+template <class S>
+__device__ __forceinline__ void put_fields(const FieldOut& out, const InstDev& I, size_t k, int y,
+                                           typename S::C cc, typename S::C clo, typename S::C p,
+                                           typename S::C T, const Drive<S>& d) {
+  if (S::kind != ST_F64 && out.f32)  // one rounding of the same sum:
+    out.put(0, k, cc + clo);         // in FP64 it is exact where it can matter
+  else
+    out.put(0, k, (double)cc + (double)clo);
+  out.put(1, k, p);
+  out.put(2, k, d.ux);
+  out.put(3, k, d.uy);
+  if constexpr (dev_h<S>())
+    out.put(4, k, (double)T + (I.hr0 + I.hr1 * y));
+  else
+    out.put(4, k, T);
+}
+
 // Velocity gradients d_x u_x, d_y u_x, d_x u_y, d_y u_y of a cell from the
 // pre-pass's u (isotropic stencil in index order; no slip: the ghost rows hold
 // minus the mirror cell's u).
@@ -363,20 +383,7 @@ struct Tile {
         return;
       }
       if (MODE == 1) {
-        // bound by the populations' load and, where it has to convert, by the
-        // FP64 pipe (64 clocks a warp instruction): floats go out as floats
-        const size_t k = (size_t)gy * nx + gx;
-        if (S::kind != ST_F64 && out.f32)  // one rounding of the same sum:
-          out.put(0, k, cc + clo);         // in FP64 it is exact where it can matter
-        else
-          out.put(0, k, (double)cc + (double)clo);
-        out.put(1, k, pcor);
-        out.put(2, k, d.ux);
-        out.put(3, k, d.uy);
-        if constexpr (dev_h<S>())
-          out.put(4, k, (double)TT + (I.hr0 + I.hr1 * gy));
-        else
-          out.put(4, k, TT);
+        put_fields<S>(out, I, (size_t)gy * nx + gx, gy, cc, clo, pcor, TT, d);
         return;
       }
 

@@ -4,9 +4,11 @@ no double can be stored at, overlapping (written in order: the last one stays)
 and on the host.  All hold the same values: FP32 is the FP64 value rounded."""
 import ctypes
 
+import numpy as np
 import pytest
 import torch
 
+from helpers import gpu_fields, oracle_fields
 from paper_1412_6238_gb300 import workloads as wl
 from paper_1412_6238_gb300.lbe import FIELD_NAMES, LBE
 
@@ -50,3 +52,29 @@ def test_outputs_hold_the_same_values(storage, nx, ny):
     raw = torch.zeros(2 * N + 1, dtype=torch.float32, device="cuda")
     export(sim, [raw.data_ptr() + 4, 0, 0, 0, 0], True, 0)
     assert torch.equal(raw[1:].cpu().view(torch.float64), full[0])
+
+
+@pytest.mark.parametrize("options", [{}, dict(interp=1, wall_mid=1, cos_wet=0.4)])
+@pytest.mark.parametrize("storage", ["f32", "f16mix", "f16dev", "bf16dev"])
+@pytest.mark.parametrize("nx,ny", [(3, 8), (4, 2), (5, 9), (127, 11), (128, 3), (129, 40),
+                                   (300, 97)])
+def test_fields_are_those_of_the_state(orc, storage, nx, ny, options):
+    """The fields of a single-precision storage (the strip kernel's, from four
+    columns on) against the oracle's of the same populations.  FP32 sums of nine
+    terms: at most 8 roundings of 6e-8 of the largest, 5e-7; c, p, T to 2e-6 of
+    their largest value.  u holds half the force, whose curvature comes from
+    differences of c near 1e-2 of it: 1e-4 of the largest |u|."""
+    def drop(nx, ny):
+        w = wl.droplet(nx, ny, max(2.0, min(nx, ny) / 4.0), nx / 2.0, ny / 2.0, Re=0.2, Ma=10.0,
+                       Ca=0.05, eta_m=0.2, eta_r=0.5, lam_r=0.5)
+        w.params.update(options)
+        return w
+    w = drop(nx, ny)
+    sim = LBE([drop(33, 12), w], storage=storage)
+    sim.step(6)
+    got = gpu_fields(sim, 1)
+    want = oracle_fields(orc, w, sim.get_state(1).numpy())
+    u = max(np.abs(want["ux"]).max(), np.abs(want["uy"]).max())
+    for k in FIELD_NAMES:
+        scale, tol = (u, 1e-4) if k in ("ux", "uy") else (np.abs(want[k]).max(), 2e-6)
+        assert np.abs(got[k] - want[k]).max() <= tol * scale, k
