@@ -59,6 +59,7 @@ struct lbe_handle {
   int seg_req = 0;               // strip kernel: rows per work item (0 = auto)
   int seg = 0;
   int* d_err = nullptr;          // device error word (strip kernel wait time-outs)
+  int* h_err = nullptr;          // its copy in pinned host memory
   uint32_t* d_seed = nullptr;    // step counter (random bits of the stochastic rounding)
   int poll_lim = STASH_POLLS;    // polls of one bounded copy wait
   int withhold = -1;             // test hook: source row whose copies are not issued
@@ -114,21 +115,23 @@ bool fault_alloc() {
   return s && strcmp(s, "alloc") == 0;
 }
 
-// Bounded wait for all work enqueued on the handle's stream so far.
+// Bounded wait for all work enqueued on the handle's stream so far.  A wait of
+// up to SPIN_US polls; a sleep of 50 us returns about 110 us later, more than
+// the fields of a 512 x 512 grid take.
+constexpr long SPIN_US = 500;
 lbe_status wait_stream(lbe_handle* h) {
   CU(h, cudaEventRecord(h->ev, h->stream));
   const auto t0 = std::chrono::steady_clock::now();
   const long lim = timeout_ms();
-  int spins = 0;
   for (;;) {
     cudaError_t e = cudaEventQuery(h->ev);
     if (e == cudaSuccess) return LBE_OK;
     if (e != cudaErrorNotReady)
       return fail(h, LBE_ECUDA, "while waiting for the stream: %s", cudaGetErrorString(e));
-    const auto ms = std::chrono::duration_cast<std::chrono::milliseconds>(
+    const auto us = std::chrono::duration_cast<std::chrono::microseconds>(
                         std::chrono::steady_clock::now() - t0).count();
-    if (ms > lim) return fail(h, LBE_ETIMEOUT, "stream not done after %ld ms", lim);
-    if (++spins > 64) std::this_thread::sleep_for(std::chrono::microseconds(50));
+    if (us / 1000 > lim) return fail(h, LBE_ETIMEOUT, "stream not done after %ld ms", lim);
+    if (us > SPIN_US) std::this_thread::sleep_for(std::chrono::microseconds(50));
   }
 }
 
@@ -149,11 +152,11 @@ lbe_status to_host(lbe_handle* h, void* dst, const void* src, size_t bytes) {
 // that ran out in any step since the word was last cleared (lbe_init,
 // lbe_set_state, lbe_load) makes every later wait report LBE_ECUDA.
 lbe_status wait(lbe_handle* h) {
-  lbe_status st = wait_stream(h);
+  if (h->d_err)
+    CU(h, cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  const lbe_status st = wait_stream(h);
   if (st || !h->d_err) return st;
-  int e = 0;
-  CU(h, cudaMemcpyAsync(&e, h->d_err, sizeof e, cudaMemcpyDeviceToHost, h->stream));
-  if ((st = wait_stream(h))) return st;
+  const int e = *h->h_err;
   if (e)
     return fail(h, LBE_ECUDA, "%s (device error word %d); the state is lost: set a state or "
                 "load a checkpoint",
@@ -344,6 +347,7 @@ void free_handle(lbe_handle* h) {
   if (h->d_inst) cudaFree(h->d_inst);
   if (h->d_pinst) cudaFree(h->d_pinst);
   if (h->d_err) cudaFree(h->d_err);
+  if (h->h_err) cudaFreeHost(h->h_err);
   if (h->d_seed) cudaFree(h->d_seed);
   if (h->d_finst) cudaFree(h->d_finst);
   if (h->scratch) cudaFree(h->scratch);
@@ -825,6 +829,7 @@ lbe_status create(int32_t n, const lbe_params* params, const lbe_init_fields* in
     CUB(e);
     CUB(es);
   }
+  CUB(cudaMallocHost(&h->h_err, sizeof(int)));
   CUB(cudaMalloc(&h->d_err, sizeof(int)));
   CUB(cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream));
   CUB(cudaMalloc(&h->d_seed, sizeof(uint32_t)));
