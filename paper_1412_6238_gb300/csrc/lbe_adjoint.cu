@@ -170,6 +170,7 @@ template <class S>
 __global__ void __launch_bounds__(256)
 state_kernel(Geo G, const InstDev* __restrict__ d, int parity, typename S::C* __restrict__ out) {
   using R = typename S::C;
+  grid_wait();
   const InstDev& I = *d;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= G.nx) return;
@@ -428,6 +429,7 @@ __global__ void __launch_bounds__(TPB, sizeof(R) == 4 ? 2 : 1)
 adjoint_A(Geo G, const InstDev* __restrict__ d, State<R> st, const R* __restrict__ a,
           const R* __restrict__ at, const double* __restrict__ obs, double wl,
           R* __restrict__ aout, R* __restrict__ S, double* __restrict__ part) {
+  grid_wait();
   extern __shared__ __align__(16) char smem_raw[];
   TileA<R>& sm = *reinterpret_cast<TileA<R>*>(smem_raw);
   StageA<R>& sg = *reinterpret_cast<StageA<R>*>(smem_raw + sizeof(TileA<R>));
@@ -722,6 +724,7 @@ template <class R>
 __global__ void __launch_bounds__(TPB)
 adjoint_B(Geo G, const InstDev* __restrict__ d, State<R> st, const R* __restrict__ S,
           R* __restrict__ tout) {
+  grid_wait();
   using Tl = TileB<R>;
   extern __shared__ __align__(16) char smem_raw[];
   Tl& sm = *reinterpret_cast<Tl*>(smem_raw);
@@ -844,8 +847,8 @@ int cell_grid(const Geo& G) {
 template <class S>
 cudaError_t state_t(const InstDev* d, const Geo& G, int parity, void* out, cudaStream_t s) {
   const dim3 grid((G.nx + 255) / 256, G.ny < 65535 ? G.ny : 65535);
-  state_kernel<S><<<grid, 256, 0, s>>>(G, d, parity, static_cast<typename S::C*>(out));
-  return cudaGetLastError();
+  return launch_early(state_kernel<S>, grid, 256, 0, s, G, d, parity,
+                      static_cast<typename S::C*>(out));
 }
 
 template <class R>
@@ -866,9 +869,10 @@ cudaError_t step_t(const InstDev* d, const Geo& G, const State<R>& st, const R* 
     if (e != cudaSuccess) return e;
     opted[dev] = true;
   }
-  adjoint_A<R><<<tiles, TPB, smem_A, s>>>(G, d, st, a, at, obs, wl, aout, S, part);
-  adjoint_B<R><<<tiles, TPB, sizeof(TileB<R>), s>>>(G, d, st, S, tout);
-  return cudaGetLastError();
+  e = launch_early(adjoint_A<R>, dim3(tiles), TPB, smem_A, s, G, d, st, a, at, obs, wl, aout, S,
+                   part);
+  if (e != cudaSuccess) return e;
+  return launch_early(adjoint_B<R>, dim3(tiles), TPB, sizeof(TileB<R>), s, G, d, st, S, tout);
 }
 
 }  // namespace adj
