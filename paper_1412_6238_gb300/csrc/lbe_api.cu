@@ -29,6 +29,7 @@ struct InstHost {
   double* walls = nullptr;  // device: Tbot[nx], Ttop[nx], then 4 float tables
   double* pcorr = nullptr;  // device [ny][nx]: corrected p (varying density only)
   double* uvel = nullptr;   // device [2][ny][nx]: u of every cell (dissipation term only)
+  void* drive = nullptr;    // device: the pre-pass's planes, instead of pcorr and uvel
   std::vector<double> Tbot, Ttop;
   std::vector<float> wdev;  // host copy of the T_w - T_r tables
 };
@@ -269,6 +270,8 @@ void fill_desc(lbe_handle* h, int j, InstDev& D) {
   P.kw = p.cos_wet * std::sqrt(2.0 * p.beta) / p.eps;
   D.pcorr = H.pcorr;
   D.uvel = H.uvel;
+  D.drive = H.drive;
+  D.dissip = H.p.dissip;
   P.eta_n2 = p.eta_n * p.eta_n;
   // divisors: the rounded reciprocal and how a quotient is formed from it
   auto den = [](double b, double& y, double& k) {
@@ -343,6 +346,7 @@ void free_handle(lbe_handle* h) {
     if (H.walls) cudaFree(H.walls);
     if (H.pcorr) cudaFree(H.pcorr);
     if (H.uvel) cudaFree(H.uvel);
+    if (H.drive) cudaFree(H.drive);
   }
   if (h->d_inst) cudaFree(h->d_inst);
   if (h->d_pinst) cudaFree(h->d_pinst);
@@ -356,6 +360,54 @@ void free_handle(lbe_handle* h) {
   if (h->ev) cudaEventDestroy(h->ev);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
+}
+
+// The shape of an FP64 handle's tiles (see SPLIT_TILE).
+int f64_shape(const lbe_handle* h) {
+  int max_nx = 0;
+  int64_t split = 0;
+  const TileShape sp = TILE_SHAPES[SPLIT_TILE];
+  for (auto& H : h->inst) {
+    max_nx = std::max(max_nx, H.nx);
+    split += (int64_t)((H.nx + sp.tx - 1) / sp.tx) * ((H.ny + sp.ty - 1) / sp.ty);
+  }
+  if (split <= (int64_t)SPLIT_PER_SM * h->num_sms) return SPLIT_TILE;
+  return max_nx <= NARROW_NX ? NARROW_TILE : F64_TILE;
+}
+
+// Planes for the pre-pass of a varying density or the dissipation term to leave
+// all it computes in, so that the pass that collides need not compute it again.
+// us a step, again / left: FP64 500 x 333 density ratio 453 / 367, dissipation
+// 490 / 413; FP32 dissipation 512 x 256 35.0 / 27.3, 1000 x 700 188 / 155; FP64
+// 128 x 128 67 / 46.  Only where every instance has a pre-pass (the others
+// would be given one), not for the split tiles, and only with room to spare: a
+// grid that barely fits keeps pcorr and uvel, and so does one whose allocation
+// fails.
+void take_drive_planes(lbe_handle* h) {
+  size_t bytes = 0, room = 0, total = 0;
+  const size_t esz = h->storage == LBE_F64 ? sizeof(double) : sizeof(float);
+  for (auto& H : h->inst) {
+    if (!H.pcorr && !H.uvel) return;
+    bytes += esz * DRIVE_NUM * (size_t)H.nx * H.ny;
+  }
+  if (h->storage == LBE_F64 && f64_shape(h) == SPLIT_TILE) return;
+  const size_t spare = sizeof(double) * 32 * (size_t)h->max_cells + ((size_t)256 << 20);
+  bool ok = cudaMemGetInfo(&room, &total) == cudaSuccess && room >= bytes + spare;
+  for (auto& H : h->inst)
+    ok = ok && cudaMalloc(&H.drive, esz * DRIVE_NUM * (size_t)H.nx * H.ny) == cudaSuccess;
+  cudaGetLastError();
+  for (int j = 0; j < h->n; j++) {
+    InstHost& H = h->inst[j];
+    if (!ok) {
+      if (H.drive) cudaFree(H.drive);
+      H.drive = nullptr;
+      continue;
+    }
+    if (H.pcorr) cudaFree(H.pcorr);
+    if (H.uvel) cudaFree(H.uvel);
+    H.pcorr = H.uvel = nullptr;
+    fill_desc(h, j, h->idev[j]);
+  }
 }
 
 // Rows per item of the strips (nc columns) of n instances: of lo..hi, the one
@@ -438,19 +490,7 @@ lbe_status setup_tiles(lbe_handle* h) {
     h->graph_failed = false;
     return wait(h);
   }
-  h->shape = h->tile;
-  if (h->storage == LBE_F64) {
-    int max_nx = 0;
-    int64_t split = 0;
-    const TileShape sp = TILE_SHAPES[SPLIT_TILE];
-    for (auto& H : h->inst) {
-      max_nx = std::max(max_nx, H.nx);
-      split += (int64_t)((H.nx + sp.tx - 1) / sp.tx) * ((H.ny + sp.ty - 1) / sp.ty);
-    }
-    h->shape = split <= (int64_t)SPLIT_PER_SM * h->num_sms ? SPLIT_TILE
-               : max_nx <= NARROW_NX                        ? NARROW_TILE
-                                                            : F64_TILE;
-  }
+  h->shape = h->storage == LBE_F64 ? f64_shape(h) : h->tile;
   const TileShape ts = TILE_SHAPES[h->shape];
   int64_t begin = 0;
   for (int j = 0; j < h->n; j++) {
@@ -508,6 +548,9 @@ cudaError_t launch_one_step(lbe_handle* h, int parity, int64_t ahead) {
     e = h->storage == LBE_F64
             ? pcorr_f64(h->d_pinst, h->n, h->p_tiles, parity, h->p_grid, h->stream)
             : pcorr_f32(h->d_pinst, h->n, h->p_tiles, parity, h->p_grid, h->stream);
+  if (e == cudaSuccess && h->inst[0].drive)
+    return h->storage == LBE_F64 ? drive_f64(h->d_pinst, h->n, h->p_tiles, parity, h->stream)
+                                 : drive_f32(h->d_pinst, h->n, h->p_tiles, parity, h->stream);
   if (e == cudaSuccess)
     e = launch_step(h->storage, h->shape, h->d_inst, h->n, h->total_tiles, parity, h->grid,
                     count, h->stream);
@@ -775,6 +818,7 @@ lbe_status create(int32_t n, const lbe_params* params, const lbe_init_fields* in
     }
     h->max_cells = std::max<int64_t>(h->max_cells, (int64_t)H.nx * H.ny);
   }
+  take_drive_planes(h);
   CUB(cudaMalloc(&h->d_inst, sizeof(InstDev) * n));
   CUB(cudaMalloc(&h->d_finst, sizeof(InstDev) * n));
   {
@@ -788,15 +832,17 @@ lbe_status create(int32_t n, const lbe_params* params, const lbe_init_fields* in
     CUB(cudaMemcpyAsync(h->d_finst, f.data(), sizeof(InstDev) * n, cudaMemcpyHostToDevice,
                         h->stream));
     if (h->vrho || h->dissip) {
-      // the pre-pass (corrected p, u): shape-0 tiles of all instances in
-      // one work list
+      // the pre-pass: tiles of all instances in one work list
+      const TileShape pre = TILE_SHAPES[pre_shape(h->storage)];
       int64_t begin = 0;
       for (auto& D : f) {
+        D.tiles_x = (D.nx + pre.tx - 1) / pre.tx;
+        D.tiles_y = (D.ny + pre.ty - 1) / pre.ty;
         D.tile_begin = begin;
         begin += (int64_t)D.tiles_x * D.tiles_y;
       }
       h->p_tiles = begin;
-      h->p_grid = (int)std::min<int64_t>(begin, (int64_t)2 * h->num_sms);
+      h->p_grid = (int)std::min<int64_t>(begin, (int64_t)4 * h->num_sms);
       CUB(cudaMalloc(&h->d_pinst, sizeof(InstDev) * n));
       CUB(cudaMemcpyAsync(h->d_pinst, f.data(), sizeof(InstDev) * n, cudaMemcpyHostToDevice,
                           h->stream));

@@ -258,6 +258,66 @@ struct Drive {
 };
 
 template <class S>
+__device__ __forceinline__ void first_moment(const typename S::C f[9], typename S::C& jx,
+                                             typename S::C& jy, typename S::C& jxl,
+                                             typename S::C& jyl) {
+  using C = typename S::C;
+  // S6 (Eq. 13): first moments.  FP64: summed in index order (the order of
+  // the FP64 reference).  FP32: differences of opposite populations first,
+  // each exact (Sterbenz: the two are within a factor 2 of each other), then
+  // their sum, so that j is rounded at its own scale; summed in index order,
+  // every partial sum is of the size of f and rounds at that scale, an error
+  // that is large next to a small j (slow flow, where f is mostly w_i p) and
+  // repeats step after step where the flow is steady.
+  jxl = jyl = C(0);
+  if constexpr (sizeof(C) == 4) {
+    // j exactly, as two floats: the three differences are exact, their sums
+    // by error-free two-sums
+    const C d13 = f[1] - f[3], d24 = f[2] - f[4], d57 = f[5] - f[7], d86 = f[8] - f[6];
+    C sx, ex, sy, ey, e2;
+    two_sum(d57, d86, sx, ex);
+    two_sum(d13, sx, jx, e2);
+    jxl = ex + e2;
+    two_sum(d57, -d86, sy, ey);
+    two_sum(d24, sy, jy, e2);
+    jyl = ey + e2;
+  } else {
+    jx = f[1] - f[3];
+    jx = jx + f[5];
+    jx = jx - f[6];
+    jx = jx - f[7];
+    jx = jx + f[8];
+    jy = f[2] - f[4];
+    jy = jy + f[5];
+    jy = jy + f[6];
+    jy = jy - f[7];
+    jy = jy - f[8];
+  }
+}
+
+// J of Drive, from the first moments and F
+template <class S>
+__device__ __forceinline__ void set_momentum(Drive<S>& d, typename S::C jx, typename S::C jy,
+                                             typename S::C jxl, typename S::C jyl) {
+  using C = typename S::C;
+  const C wa = WGT<C>(1), wd2 = C(2) * WGT<C>(5);
+  if constexpr (sizeof(C) == 4) {
+    // J = j + (w_axis + 2 w_diag) F as two floats (the force term, small
+    // next to j where the momentum matters, is rounded at its own scale)
+    const C cFx = fmaf(wa, d.Fx, wd2 * d.Fx), cFy = fmaf(wa, d.Fy, wd2 * d.Fy);
+    C e;
+    two_sum(jx, cFx, d.Jx, e);
+    d.Jxl = e + jxl;
+    two_sum(jy, cFy, d.Jy, e);
+    d.Jyl = e + jyl;
+  } else {
+    d.Jx = (jx + wa * d.Fx) + wd2 * d.Fx;
+    d.Jy = (jy + wa * d.Fy) + wd2 * d.Fy;
+    d.Jxl = d.Jyl = C(0);
+  }
+}
+
+template <class S>
 __device__ __forceinline__ Drive<S> drive(const Phys<typename S::C>& P, int gy,
                                           const typename S::C f[9], typename S::C cc,
                                           typename S::C TT, const Stencils<typename S::C>& s) {
@@ -283,55 +343,12 @@ __device__ __forceinline__ Drive<S> drive(const Phys<typename S::C>& P, int gy,
   d.dRy = vr ? (cs2<C>() * P.drho) * s.gcy : C(0);
   d.Fx = cap * s.gcx + mar * (g2 * s.gTx - cdT * s.gcx) + (vr ? d.rho * P.ax : P.Fbx);
   d.Fy = cap * s.gcy + mar * (g2 * s.gTy - cdT * s.gcy) + (vr ? d.rho * P.ay : P.Fby);
-  // S6 (Eq. 13): first moments.  FP64: summed in index order (the order of
-  // the FP64 reference).  FP32: differences of opposite populations first,
-  // each exact (Sterbenz: the two are within a factor 2 of each other), then
-  // their sum, so that j is rounded at its own scale; summed in index order,
-  // every partial sum is of the size of f and rounds at that scale, an error
-  // that is large next to a small j (slow flow, where f is mostly w_i p) and
-  // repeats step after step where the flow is steady.
-  C jx, jy, jxl = C(0), jyl = C(0);
-  if constexpr (sizeof(C) == 4) {
-    // j exactly, as two floats: the three differences are exact, their sums
-    // by error-free two-sums
-    const C d13 = f[1] - f[3], d24 = f[2] - f[4], d57 = f[5] - f[7], d86 = f[8] - f[6];
-    C sx, ex, sy, ey, e2;
-    two_sum(d57, d86, sx, ex);
-    two_sum(d13, sx, jx, e2);
-    jxl = ex + e2;
-    two_sum(d57, -d86, sy, ey);
-    two_sum(d24, sy, jy, e2);
-    jyl = ey + e2;
-  } else {
-    jx = f[1] - f[3];
-    jx = jx + f[5];
-    jx = jx - f[6];
-    jx = jx - f[7];
-    jx = jx + f[8];
-    jy = f[2] - f[4];
-    jy = jy + f[5];
-    jy = jy + f[6];
-    jy = jy - f[7];
-    jy = jy - f[8];
-  }
+  C jx, jy, jxl, jyl;
+  first_moment<S>(f, jx, jy, jxl, jyl);
   const Dens<C> dn = make_dens(P, d.rho, vr);
   d.ux = dv(jx, dn.rcs2) + dv(C(0.5) * d.Fx, dn.rho);
   d.uy = dv(jy, dn.rcs2) + dv(C(0.5) * d.Fy, dn.rho);
-  const C wa = WGT<C>(1), wd2 = C(2) * WGT<C>(5);
-  if constexpr (sizeof(C) == 4) {
-    // J = j + (w_axis + 2 w_diag) F as two floats (the force term, small
-    // next to j where the momentum matters, is rounded at its own scale)
-    const C cFx = fmaf(wa, d.Fx, wd2 * d.Fx), cFy = fmaf(wa, d.Fy, wd2 * d.Fy);
-    C e;
-    two_sum(jx, cFx, d.Jx, e);
-    d.Jxl = e + jxl;
-    two_sum(jy, cFy, d.Jy, e);
-    d.Jyl = e + jyl;
-  } else {
-    d.Jx = (jx + wa * d.Fx) + wd2 * d.Fx;
-    d.Jy = (jy + wa * d.Fy) + wd2 * d.Fy;
-    d.Jxl = d.Jyl = C(0);
-  }
+  set_momentum<S>(d, jx, jy, jxl, jyl);
   return d;
 }
 

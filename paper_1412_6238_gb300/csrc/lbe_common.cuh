@@ -142,6 +142,11 @@ struct FieldOut {
 #endif
 };
 
+// Planes of InstDev::drive: what the pre-pass of a varying density or of the
+// dissipation term leaves to the pass that collides.
+enum { DRIVE_C, DRIVE_T, DRIVE_MU, DRIVE_FX, DRIVE_FY, DRIVE_GX, DRIVE_GY, DRIVE_P, DRIVE_UX,
+       DRIVE_UY, DRIVE_NUM };
+
 // The number of a step: a handle's counter in device memory (the steps before
 // the current group of launches) and the step's place in the group, so that
 // the counter is advanced once per group and a captured group can be replayed.
@@ -170,6 +175,7 @@ __device__ __forceinline__ void grid_release() {
 struct InstDev {
   int32_t nx, ny, pitch, tiles_x;
   int32_t tiles_y, storage;
+  int32_t dissip;       // the dissipation term is on
   int64_t tile_begin;   // first global tile / work-item index of this instance
   uint64_t plane_bytes; // bytes between consecutive planes
   uint64_t g0_off;      // byte offset of the FP32 g_0 plane (16-bit forms)
@@ -190,6 +196,7 @@ struct InstDev {
   uint32_t salt;        // the instance's index in its handle (random bits)
   double* pcorr;        // varying density: p of Eq. 13 with its correction, [ny][nx]
   double* uvel;         // dissipation term: u of every cell, [2][ny][nx] (FP64)
+  void* drive;          // the pre-pass's results, planes of the storage's type (see DRIVE_*)
 };
 
 template <class C>

@@ -46,6 +46,8 @@ constexpr int SPLIT_PER_SM = 2;
 constexpr TileShape TILE_SHAPES[NUM_TILES + 3] = {{32, 8},  {64, 4},  {32, 16}, {64, 8},
                                                   {128, 4}, {124, 0}, {60, 0},  {128, 0},
                                                   {128, 0}, {4, 8},   {16, 8},  {4, 8}};
+// The tiles of the pre-pass (and of the pass that collides after it).
+constexpr int pre_shape(int storage) { return storage == ST_F64 ? F64_TILE : 0; }
 inline bool is_strip(int tile) { return tile >= STRIP_FIRST && tile < NUM_TILES; }
 inline bool is_stash(int tile) { return tile == STASH_ID || tile == STASH_OWN_ID; }
 
@@ -157,12 +159,15 @@ int occupancy_mix(int tile);
 cudaError_t fields_f64(const InstDev* d, int64_t tiles, int parity, const FieldOut& out,
                        cudaStream_t s);
 // Varying density (FP64 storage only): the corrected p of Eq. 13 of every
-// cell into each instance's pcorr; d is a work list of tile shape 0.
+// cell into each instance's pcorr (or drive); d is a work list of pre_shape.
 cudaError_t pcorr_f64(const InstDev* d, int n, int64_t total, int parity, int grid,
                       cudaStream_t s);
 // FP32 storage: the pre-pass of the dissipation term (u of every cell)
 cudaError_t pcorr_f32(const InstDev* d, int n, int64_t total, int parity, int grid,
                       cudaStream_t s);
+// The pass that collides, after a pre-pass into every instance's `drive`.
+cudaError_t drive_f64(const InstDev* d, int n, int64_t total, int parity, cudaStream_t s);
+cudaError_t drive_f32(const InstDev* d, int n, int64_t total, int parity, cudaStream_t s);
 cudaError_t fields_f32(const InstDev* d, int64_t tiles, int parity, const FieldOut& out,
                        cudaStream_t s);
 cudaError_t fields_f16(const InstDev* d, int64_t tiles, int parity, const FieldOut& out,

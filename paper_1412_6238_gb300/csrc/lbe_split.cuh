@@ -151,7 +151,7 @@ struct SplitTile {
     const C cc = c0[tx + 2], pp = sm.p[qo + tx + 1], TT = sm.T[qo + tx + 1];
     const Drive<S> d = drive<S>(P, gy, f, cc, TT, st);
     C du[4];
-    if (I.uvel != nullptr) grad_u(I, gx, gy, du);
+    if (I.uvel != nullptr) grad_u(nx, ny, I.uvel, gx, gy, du);
     const C* wdu = I.uvel != nullptr ? du : nullptr;
     char* __restrict__ dst = I.buf[parity ^ 1];
     if (warp == 0)

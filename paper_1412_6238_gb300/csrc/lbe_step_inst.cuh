@@ -79,14 +79,24 @@ int LBE_CAT(occupancy_, LBE_SUFFIX)(int tile) {
 }
 
 #if LBE_PCORR
-// Varying density: the corrected p of every cell of every instance into its
-// pcorr (tiles of shape 0 over a work list of that shape), before the step.
+// The pre-pass of a varying density or the dissipation term, over a work list of
+// tiles of PRE_SHAPE, and the pass that collides from what it left in `drive`.
+namespace {
+constexpr TileShape PRE = TILE_SHAPES[pre_shape(LBE_ST::kind)];
+}
 cudaError_t LBE_CAT(pcorr_, LBE_SUFFIX)(const InstDev* d, int n, int64_t total, int parity,
                                          int grid, cudaStream_t s) {
   if (grid <= 0) grid = 1;
   if ((int64_t)grid > total) grid = (int)total;
-  return launch_early(tile_kernel<LBE_ST, 32, 8, 2>, dim3(grid), 256, 0, s, d, n, total, parity,
+  return launch_early(tile_kernel<LBE_ST, PRE.tx, PRE.ty, 2>, dim3(grid), PRE.tx * PRE.ty, 0, s, d, n, total, parity,
                       FieldOut{}, StepCount{});
+}
+cudaError_t LBE_CAT(drive_, LBE_SUFFIX)(const InstDev* d, int n, int64_t total, int parity,
+                                         cudaStream_t s) {
+  const int64_t parts = total * (PRE.tx * PRE.ty / DRIVE_THREADS);
+  return launch_early(drive_kernel<LBE_ST, PRE.tx, PRE.ty>,
+                      dim3((unsigned)std::min<int64_t>(parts, 2147483647)), DRIVE_THREADS, 0, s, d,
+                      n, total, parity);
 }
 #endif
 

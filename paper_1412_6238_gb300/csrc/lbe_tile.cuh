@@ -212,11 +212,10 @@ __device__ __forceinline__ void put_fields(const FieldOut& out, const InstDev& I
 }
 
 // Velocity gradients d_x u_x, d_y u_x, d_x u_y, d_y u_y of a cell from the
-// pre-pass's u (isotropic stencil in index order; no slip: the ghost rows hold
-// minus the mirror cell's u).
-template <class C>
-__device__ __forceinline__ void grad_u(const InstDev& I, int gx, int gy, C du[4]) {
-  const int nx = I.nx, ny = I.ny;
+// pre-pass's u, two planes (isotropic stencil in index order; no slip: the
+// ghost rows hold minus the mirror cell's u).
+template <class C, class U>
+__device__ __forceinline__ void grad_u(int nx, int ny, const U* u, int gx, int gy, C du[4]) {
   const size_t N = (size_t)nx * ny;
   C s0 = C(0), s1 = C(0), s2 = C(0), s3 = C(0);
   for (int i = 1; i < 9; i++) {
@@ -231,7 +230,7 @@ __device__ __forceinline__ void grad_u(const InstDev& I, int gx, int gy, C du[4]
       sg = C(-1);
     }
     const size_t kk = (size_t)yy * nx + xx;
-    const C vx = sg * (C)I.uvel[kk], vy = sg * (C)I.uvel[N + kk];
+    const C vx = sg * (C)u[kk], vy = sg * (C)u[N + kk];
     s0 += WGT<C>(i) * C(EX(i)) * vx;
     s1 += WGT<C>(i) * C(EY(i)) * vx;
     s2 += WGT<C>(i) * C(EX(i)) * vy;
@@ -278,7 +277,7 @@ struct Tile {
     // density (pcorr) or the dissipation term (uvel); the whole CTA leaves
     // together
     const bool wants_p = nonzero(P.drho) && I.pcorr != nullptr;
-    if (MODE == 2 && !wants_p && I.uvel == nullptr) return;
+    if (MODE == 2 && !wants_p && I.uvel == nullptr && I.drive == nullptr) return;
 
     // ---- S1: own cell
     const int gx = x0 + tx, gy = y0 + ty;
@@ -375,6 +374,21 @@ struct Tile {
       const C pcor = nonzero(P.drho) ? pp + C(0.5) * (d.ux * d.dRx + d.uy * d.dRy) : pp;
       if (MODE == 2) {  // the corrected p and u for the step that follows
         const size_t k = (size_t)gy * nx + gx;
+        if (I.drive != nullptr) {
+          C* const o = static_cast<C*>(I.drive) + k;
+          const size_t N = (size_t)nx * ny;
+          o[DRIVE_C * N] = cc;
+          o[DRIVE_T * N] = TT;
+          o[DRIVE_MU * N] = d.mu;
+          o[DRIVE_FX * N] = d.Fx;
+          o[DRIVE_FY * N] = d.Fy;
+          o[DRIVE_GX * N] = st.gcx;
+          o[DRIVE_GY * N] = st.gcy;
+          o[DRIVE_P * N] = pcor;
+          o[DRIVE_UX * N] = d.ux;
+          o[DRIVE_UY * N] = d.uy;
+          return;
+        }
         if (wants_p) I.pcorr[k] = (double)pcor;
         if (I.uvel) {
           I.uvel[k] = (double)d.ux;
@@ -397,7 +411,7 @@ struct Tile {
       C gs = C(0);  // 16-bit forms: the stored moving g_i
       // the dissipation term
       C du[4] = {C(0), C(0), C(0), C(0)};
-      if (I.uvel != nullptr) grad_u(I, gx, gy, du);
+      if (I.uvel != nullptr) grad_u(nx, ny, I.uvel, gx, gy, du);
       collide<S>(P, f, g, h, cc, pp, TT, st.gpx, st.gpy, d,
                  [&](int k, int i, C v) {
                    if constexpr (S::SR) {
@@ -442,6 +456,84 @@ tile_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_tiles, 
     const InstDev& I = insts[lo];
     T::run(I, t - I.tile_begin, parity, sm, out, step);
     __syncthreads();
+  }
+}
+
+// The step of cells whose moments, force and u the pre-pass has left in
+// I.drive: grad p, and the collisions.  One cell a thread; nothing is shared, so
+// CTAs of DRIVE_THREADS take the tiles of the pre-pass's work list in parts.
+constexpr int DRIVE_THREADS = 128;
+template <class S, int TX, int TY>
+__global__ void __launch_bounds__(DRIVE_THREADS, S::kind == ST_F64 ? 1 : 4)
+drive_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_tiles, int parity) {
+  using C = typename S::C;
+  static_assert(!S::SR, "no stochastic rounding here");
+  constexpr int PARTS = TX * TY / DRIVE_THREADS, ROWS = TY / PARTS;
+  grid_wait();
+  for (int64_t t = blockIdx.x; t < PARTS * total_tiles; t += gridDim.x) {
+    int lo = 0, hi = n_inst - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (insts[mid].tile_begin <= t / PARTS) lo = mid; else hi = mid - 1;
+    }
+    const InstDev& I = insts[lo];
+    const int64_t tile = t / PARTS - I.tile_begin;
+    const int nx = I.nx, ny = I.ny;
+    const int x = (int)(tile % I.tiles_x) * TX + (int)threadIdx.x % TX;
+    const int y = (int)(tile / I.tiles_x) * TY + (int)(t % PARTS) * ROWS +
+                  (int)threadIdx.x / TX;
+    if (x >= nx || y >= ny) continue;
+    const char* __restrict__ src = I.buf[parity];
+    char* __restrict__ dst = I.buf[parity ^ 1];
+    const Phys<C> P = phys<C>(I);
+    const size_t N = (size_t)nx * ny, k = (size_t)y * nx + x, rowbase = (size_t)y * I.pitch;
+    const C* __restrict__ w = static_cast<const C*>(I.drive);
+    const Cell<S> q = make_cell<S>(x, y, nx);
+    C f[9], g[9], h[9];
+    C cc = w[DRIVE_C * N + k], g0lo = C(0), clo = C(0);
+    pull9<S, 0>(I, P, src, q, f);
+    pull9<S, 1>(I, P, src, q, g);
+    if constexpr (S::kind != ST_F64) {
+      g0lo = ld_g0lo<S>(I, src, rowbase + XG + x);
+      cc = moment_c(g, g0lo, clo);
+    }
+    const bool vr = sizeof(C) == 8 && nonzero(P.drho);
+    Drive<S> d;
+    d.rho = vr ? rho_at(P, cc) : P.rho;
+    pull9<S, 2, true>(I, P, src, q, h, vr ? d.rho : P.rho);
+    d.Trow = dev_h<S>() ? P.hr0 + P.hr1 * C(y) : C(0);
+    d.mu = w[DRIVE_MU * N + k];
+    d.Fx = w[DRIVE_FX * N + k];
+    d.Fy = w[DRIVE_FY * N + k];
+    d.ux = w[DRIVE_UX * N + k];
+    d.uy = w[DRIVE_UY * N + k];
+    d.dRx = vr ? (cs2<C>() * P.drho) * w[DRIVE_GX * N + k] : C(0);
+    d.dRy = vr ? (cs2<C>() * P.drho) * w[DRIVE_GY * N + k] : C(0);
+    C jx, jy, jxl, jyl;  // (FP64: unused)
+    first_moment<S>(f, jx, jy, jxl, jyl);
+    set_momentum<S>(d, jx, jy, jxl, jyl);
+    // p of the neighbours: x wraps, the ghost rows mirror
+    C p[3][3];
+    const C* __restrict__ wp = w + DRIVE_P * N;
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+      const int yy = y - 1 + j;
+      const C* r = wp + (size_t)(yy < 0 ? 0 : yy >= ny ? ny - 1 : yy) * nx;
+      p[j][0] = r[q.xm];
+      p[j][1] = r[q.x];
+      p[j][2] = r[q.xp];
+    }
+    C gpx, gpy;
+    grad3(p[0], p[1], p[2], 1, gpx, gpy);
+    C du[4];
+    const bool dis = I.dissip != 0;
+    if (dis) grad_u(nx, ny, w + DRIVE_UX * N, x, y, du);
+    C lo_out = C(0);
+    collide<S>(
+        P, f, g, h, cc, p[1][1], w[DRIVE_T * N + k], gpx, gpy, d,
+        [&](int l, int i, C v) { st_cell<S>(I, dst, l, i, rowbase, x, v); }, g0lo, clo, &lo_out,
+        (y > 0 && y < ny - 1) ? P.dh : C(0), dis ? du : nullptr);
+    if constexpr (S::kind != ST_F64) st_cell_g0lo<S>(I, dst, rowbase, x, (float)lo_out);
   }
 }
 
