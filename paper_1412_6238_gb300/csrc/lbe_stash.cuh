@@ -794,7 +794,7 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
     grid_wait();
     grid_release();
     // the step number (random bits of the stochastic rounding)
-    const uint32_t skey = S::SR ? sr_step_key(seed.now(), I.salt) : 0u;
+    const uint32_t skey = S::SR && !EXPORT ? sr_step_key(seed.now(), I.salt) : 0u;
 
     issue(ya - 2, false);
     // ring offsets of rows i - 2 .. i + 2, rotated from row to row
