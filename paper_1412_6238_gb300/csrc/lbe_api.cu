@@ -639,11 +639,19 @@ lbe_status ensure_scratch(lbe_handle* h) {
   return LBE_OK;
 }
 
+// Cells from which the fields of a single-precision storage come from the strip
+// kernel's marching rows: 4096 x 4096 FP32 0.49 ms, by the tile kernel (which
+// pulls a ring of 2/3 of a tile's cells besides) 1.79; 2048 x 2048 F16DEV 0.17,
+// 0.48.  The tile kernel takes c of that ring as a single sum, the strip kernel
+// every c in two floats, as the step does; both are as close to the FP64 fields,
+// but in the u of a flow that has hardly begun, which is the difference of two
+// nearly equal terms, they differ by up to 2.4e-5 of it (a planar layer of a few
+// ten thousand cells in 16 bits).  Smaller grids, whose fields take 50 us either
+// way, keep the tile kernel and with it every bit they had.
+constexpr int64_t STRIP_FIELDS_FROM = (int64_t)1 << 21;
 lbe_status compute_fields(lbe_handle* h, int j, int which_parity, const FieldOut& out) {
   const InstHost& H = h->inst[j];
-  if (h->storage != LBE_F64 && H.nx >= XG) {
-    // the strip kernel's marching rows: 4096 x 4096 FP32 0.49 ms, the tile
-    // kernel (which pulls a ring of 2/3 of a tile's cells besides) 1.79
+  if (h->storage != LBE_F64 && H.nx >= XG && (int64_t)H.nx * H.ny >= STRIP_FIELDS_FROM) {
     const int nc = TILE_SHAPES[STASH_ID].tx;
     const int occ = stash_occupancy(h->storage);
     if (occ <= 0) return fail(h, LBE_ECUDA, "the field kernel cannot be resident");

@@ -59,8 +59,7 @@ def test_outputs_hold_the_same_values(storage, nx, ny):
 @pytest.mark.parametrize("nx,ny", [(3, 8), (4, 2), (5, 9), (127, 11), (128, 3), (129, 40),
                                    (300, 97)])
 def test_fields_are_those_of_the_state(orc, storage, nx, ny, options):
-    """The fields of a single-precision storage (the strip kernel's, from four
-    columns on) against the oracle's of the same populations.  FP32 sums of nine
+    """The fields of a single-precision storage against the oracle's of the same populations.  FP32 sums of nine
     terms: at most 8 roundings of 6e-8 of the largest, 5e-7; c, p, T to 2e-6 of
     their largest value.  u holds half the force, whose curvature comes from
     differences of c near 1e-2 of it: 1e-4 of the largest |u|."""
@@ -74,6 +73,27 @@ def test_fields_are_those_of_the_state(orc, storage, nx, ny, options):
     sim.step(6)
     got = gpu_fields(sim, 1)
     want = oracle_fields(orc, w, sim.get_state(1).numpy())
+    u = max(np.abs(want["ux"]).max(), np.abs(want["uy"]).max())
+    for k in FIELD_NAMES:
+        scale, tol = (u, 1e-4) if k in ("ux", "uy") else (np.abs(want[k]).max(), 2e-6)
+        assert np.abs(got[k] - want[k]).max() <= tol * scale, k
+
+
+@pytest.mark.parametrize("nx,ny,options", [(4, 524299, {}), (2051, 1031, {}),
+                                           (131, 16103, dict(interp=1, wall_mid=1, cos_wet=0.4))])
+@pytest.mark.parametrize("storage", ["f32", "f16mix", "f16dev", "bf16dev"])
+def test_fields_of_large_grids(orc, storage, nx, ny, options):
+    """The same, with drops of the same sizes and the same bounds, from the number
+    of cells on where the strip kernel writes the fields (sigma varying from wall
+    to wall as in a grid of 20 rows)."""
+    assert nx * ny >= 1 << 21
+    w = wl.droplet(nx, ny, max(2.0, min(nx, 40) / 4.0), nx / 2.0, ny / 2.0, Re=0.2, Ma=10.0,
+                   Ca=0.05, eta_m=0.2, eta_r=0.5, lam_r=0.5)
+    w.params.update(options, sigmaT=w.params["sigmaT"] * 20 / ny)
+    sim = LBE([w], storage=storage)
+    sim.step(6)
+    got = gpu_fields(sim, 0)
+    want = oracle_fields(orc, w, sim.get_state(0).numpy())
     u = max(np.abs(want["ux"]).max(), np.abs(want["uy"]).max())
     for k in FIELD_NAMES:
         scale, tol = (u, 1e-4) if k in ("ux", "uy") else (np.abs(want[k]).max(), 2e-6)
