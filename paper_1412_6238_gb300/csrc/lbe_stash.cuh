@@ -705,8 +705,13 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
     char* __restrict__ dst = I.buf[parity ^ 1];
     // the instance's constants, from shared memory where they are used (held
     // in registers over the row loop they made the loop spill)
+    // The 16-bit pair forms hold the constants in registers: which products are
+    // fused with a sum depends on where the constants come from, and a stored
+    // value then rounds stochastically the other way now and then.
+    constexpr bool REG = W16 && !VAR;
+    const Phys<C> P_reg = phys<C>(I);
     auto params = [&]() {
-      Phys<C> P = s_phys;
+      Phys<C> P = REG ? P_reg : s_phys;
       if constexpr (!VAR) {  // the variants are off: known to the compiler
         P.harm = C(0);
         P.wmid = C(0);
@@ -1048,7 +1053,7 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
         const C* cc2 = cring + o2;
         auto normal = [&](int j) {
           C gx, gy;
-          normal3(ca, cb, cc2, j + 2, s_phys.eta_n2, nxr[nr(mn) + j + 2], nyr[nr(mn) + j + 2], gx,
+          normal3(ca, cb, cc2, j + 2, (REG ? P_reg : s_phys).eta_n2, nxr[nr(mn) + j + 2], nyr[nr(mn) + j + 2], gx,
                   gy);
         };
         if (!helper) normal(t);
