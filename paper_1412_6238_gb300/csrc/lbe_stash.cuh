@@ -61,6 +61,8 @@
 // row run out with nothing in flight.
 #pragma once
 
+#include <type_traits>
+
 #include "lbe_tile.cuh"
 
 namespace lbe {
@@ -212,11 +214,7 @@ struct StashCfg {
   static_assert(NC % 32 == 0, "whole warps");
 };
 
-// The 9 pulled populations of lattice K at row y from a stash slot
-// (thread t reads element t + 2 - xi_ix of population (K, i), or t + 2 where
-// the wall substitution copied the reversed population of the cell itself),
-// with the rules of pull9 (lbe_tile.cuh): anti-bounce-back for hbar at the
-// walls, and the deviation offsets of hbar between rows.
+// Population (k, i) of element col of a row of a stash slot.
 template <class S>
 __device__ __forceinline__ float stash_val(const char* slot, int k, int i, int col,
                                            const Phys<float>& P) {
@@ -231,16 +229,37 @@ __device__ __forceinline__ float stash_val(const char* slot, int k, int i, int c
   }
 }
 
-// The 9 pulled populations of lattice K at row y from a stash slot.
-// c0 is the element of the thread's own column in a population row (c0g in the
-// FP32 g_0 row of the 16-bit forms); the pull reads c0 - xi_ix, or c0 where
-// the wall substitution copied the reversed population of the cell itself.
-// Rules of pull9 (lbe_tile.cuh): anti-bounce-back for hbar at the walls, and
-// the deviation offsets of hbar between rows.
-// RAW: in an interior row, the hbar deviations as stored, relative to their
-// source rows' T_r, without the offsets +-w_i dh to this row's T_r: they
-// cancel exactly in the moment, and collide() applies them through its
-// source term.
+// Where hbar is pulled for: the collision, the moments of a column of the
+// strip, the moments of a halo column.
+enum PullFor { FOR_COLLISION, FOR_MOMENTS, FOR_HALO };
+// The rounding of a wall row's hbar, fixed here (a contraction left to the
+// compiler depends on whether it holds rho c_v dh in a register or reads it from
+// shared memory, and a 16-bit value next to a tie then rounds the other way: a
+// state would not go on bit for bit under the next build).  Bit i: w_i dh enters
+// the row change of direction i by a fused multiply-add, else rounded; bit 0:
+// so does 2 w_i rho c_v T_w in the links.  Which, is by the kernels the first
+// states were made with; the error is 2^-24 of a deviation either way.
+template <class S, bool VAR>
+__host__ __device__ constexpr unsigned wall_fma(PullFor site) {
+  constexpr unsigned ALL = 0x1ffu;
+  if (S::kind == ST_F32) return ALL;
+  if (S::kind == ST_F16MIX)
+    return VAR ? ALL : site == FOR_MOMENTS ? 1u << 2 | 1u << 4 : 1u << 4;
+  const unsigned down = 1u << 4 | 1u << 7 | 1u << 8;
+  return 1u | (VAR || site == FOR_COLLISION ? down : 0u);
+}
+// hbar of direction i of a wall row from the stored value v: of a link (wall),
+// X = 2 w_i rho c_v and T_w its temperature, or of the row next to it
+template <unsigned FMA>
+__device__ __forceinline__ float link_h(float v, float X, float Tw) {
+  return (FMA & 1u) ? fmaf(X, Tw, -v) : __fsub_rn(__fmul_rn(X, Tw), v);
+}
+template <unsigned FMA>
+__device__ __forceinline__ float row_change_h(int i, float v, float dh) {
+  const float w = EY(i) == 1 ? -WGT<float>(i) : WGT<float>(i);
+  return (FMA >> i & 1u) ? fmaf(w, dh, v) : __fadd_rn(v, __fmul_rn(w, dh));
+}
+
 // The wall temperature of the anti-bounce-back link of population i at
 // column xw (Tw: the wall temperature at xw): with P.wmid, where the link
 // crosses the wall, x - xi_ix/2, between the two columns.
@@ -253,44 +272,34 @@ __device__ __forceinline__ float link_T(const InstDev& I, const Phys<float>& P, 
   return 0.5f * (Tw + wall_T<S>(I, xs, which));
 }
 
-template <class S, int K, bool RAW = false>
-__device__ __forceinline__ void wstash_pull(const InstDev& I, const Phys<float>& P,
-                                            const char* slot, int c0, int c0g, int y, int xw,
-                                            float out[9]) {
-  constexpr bool DEV = (K == 2) && dev_h<S>();
+// The 9 pulled hbar at row y from a stash slot, with the rules of pull9
+// (lbe_tile.cuh): anti-bounce-back at the walls, and the change of reference row
+// in the rows next to them.  c0 is the element of the thread's own column in a
+// population row; the pull reads c0 - xi_ix, or c0 where the wall substitution
+// copied the reversed population of the cell itself.  In an interior row the
+// deviations are as stored, relative to their source rows' T_r, without the
+// offsets +-w_i dh to this row's T_r: they cancel exactly in the moment, and
+// collide() applies them through its source term.
+template <class S, unsigned FMA>
+__device__ __forceinline__ void wstash_pull_h(const InstDev& I, const Phys<float>& P,
+                                              const char* slot, int c0, int y, int xw,
+                                              float out[9]) {
   const bool wb = (y == 0), wt = (y == I.ny - 1);
-  auto col = [&](int i, bool shift) {
-    const int base = (K == 1 && i == 0) ? c0g : c0;
-    return shift ? base - EX(i) : base;
-  };
   if (!wb && !wt) {
-    // interior row: constant offsets
 #pragma unroll
-    for (int i = 0; i < 9; i++) {
-      float v = stash_val<S>(slot, K, i, col(i, true), P);
-      if (DEV && !RAW && EY(i) == 1) v -= WGT<float>(i) * P.dh;
-      if (DEV && !RAW && EY(i) == -1) v += WGT<float>(i) * P.dh;
-      out[i] = v;
-    }
+    for (int i = 0; i < 9; i++) out[i] = stash_val<S>(slot, 2, i, c0 - EX(i), P);
     return;
   }
-  float Tw = 0.f;
-  if (K == 2) Tw = wall_T<S>(I, xw, wb ? 0 : 1);
-  const float dh = DEV ? P.dh : 0.f;
+  const float Tw = wall_T<S>(I, xw, wb ? 0 : 1);
 #pragma unroll
   for (int i = 0; i < 9; i++) {
     const bool wall = (EY(i) == 1 && wb) || (EY(i) == -1 && wt);
-    float v = wall ? stash_val<S>(slot, K, i, col(i, false), P)
-                   : stash_val<S>(slot, K, i, col(i, true), P);
-    if (K == 2) {
-      if (wall) {
-        v = -v + 2.f * WGT<float>(i) * P.rho * P.cv * link_T<S>(I, P, xw, i, wb ? 0 : 1, Tw);
-      } else if (DEV && EY(i) == 1) {
-        v -= WGT<float>(i) * dh;
-      } else if (DEV && EY(i) == -1) {
-        v += WGT<float>(i) * dh;
-      }
-    }
+    float v = stash_val<S>(slot, 2, i, wall ? c0 : c0 - EX(i), P);
+    if (wall)
+      v = link_h<FMA>(v, 2.f * WGT<float>(i) * P.rho * P.cv,
+                      link_T<S>(I, P, xw, i, wb ? 0 : 1, Tw));
+    else if (EY(i) != 0)
+      v = row_change_h<FMA>(i, v, P.dh);
     out[i] = v;
   }
 }
@@ -345,10 +354,9 @@ __device__ __forceinline__ void wstash_pull_fg16(const InstDev& I, const Phys<fl
 
 // F16MIX: f_i, g_i and hbar_i of a pulled cell with one 8-byte load (the
 // three follow the same neighbour, and the same wall rule but for the
-// anti-bounce-back of hbar), with the rules of pull9 (lbe_tile.cuh) for
-// hbar; g_0 from the FP32 row and its low part from word 0.  c0: the
-// thread's own column in a row.  RAW: as in wstash_pull.
-template <bool RAW>
+// anti-bounce-back of hbar), hbar as wstash_pull_h; g_0 from the FP32 row and
+// its low part from word 0.  c0: the thread's own column in a row.
+template <unsigned FMA>
 __device__ __forceinline__ void wstash_pull_mix(const InstDev& I, const Phys<float>& P,
                                                 const char* slot, int c0, int y, int xw,
                                                 float f[9], float g[9], float h[9],
@@ -377,10 +385,7 @@ __device__ __forceinline__ void wstash_pull_mix(const InstDev& I, const Phys<flo
       const float2 q = two(v.y);
       f[i] = __uint_as_float(v.x);
       g[i] = q.x * sg;
-      float hv = q.y * sh;
-      if (!RAW && EY(i) == 1) hv -= WGT<float>(i) * P.dh;
-      if (!RAW && EY(i) == -1) hv += WGT<float>(i) * P.dh;
-      h[i] = hv;
+      h[i] = q.y * sh;
     }
     return;
   }
@@ -393,13 +398,11 @@ __device__ __forceinline__ void wstash_pull_mix(const InstDev& I, const Phys<flo
     f[i] = __uint_as_float(v.x);
     g[i] = q.x * sg;
     float hv = q.y * sh;
-    if (wall) {
-      hv = -hv + 2.f * WGT<float>(i) * P.rho * P.cv * link_T<StMix>(I, P, xw, i, wb ? 0 : 1, Tw);
-    } else if (EY(i) == 1) {
-      hv -= WGT<float>(i) * P.dh;
-    } else if (EY(i) == -1) {
-      hv += WGT<float>(i) * P.dh;
-    }
+    if (wall)
+      hv = link_h<FMA>(hv, 2.f * WGT<float>(i) * P.rho * P.cv,
+                       link_T<StMix>(I, P, xw, i, wb ? 0 : 1, Tw));
+    else if (EY(i) != 0)
+      hv = row_change_h<FMA>(i, hv, P.dh);
     h[i] = hv;
   }
 }
@@ -602,6 +605,7 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
   using C = float;
   constexpr bool W16 = sizeof(typename Fmt::E) == 2;
   constexpr bool MIX = S::kind == ST_F16MIX;
+  constexpr unsigned FMA_C = wall_fma<S, VAR>(FOR_COLLISION);
   extern __shared__ __align__(128) char smem[];
   constexpr int CW = Cfg::CW;
   // ring entry of column x0 + j: j + 2
@@ -705,13 +709,8 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
     char* __restrict__ dst = I.buf[parity ^ 1];
     // the instance's constants, from shared memory where they are used (held
     // in registers over the row loop they made the loop spill)
-    // The 16-bit pair forms hold the constants in registers: which products are
-    // fused with a sum depends on where the constants come from, and a stored
-    // value then rounds stochastically the other way now and then.
-    constexpr bool REG = W16 && !VAR;
-    const Phys<C> P_reg = phys<C>(I);
     auto params = [&]() {
-      Phys<C> P = REG ? P_reg : s_phys;
+      Phys<C> P = s_phys;
       if constexpr (!VAR) {  // the variants are off: known to the compiler
         P.harm = C(0);
         P.wmid = C(0);
@@ -827,14 +826,14 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
         // hbar as pulled (without the change of reference row in interior
         // rows, which collide() applies through the source term)
         if constexpr (MIX) {
-          wstash_pull_mix<true>(I, P, s, c0, r, x, f, g, h, g0lo);
+          wstash_pull_mix<FMA_C>(I, P, s, c0, r, x, f, g, h, g0lo);
         } else {
           if constexpr (!W16) {
             wstash_pull_fg(I, s, c0, r, f, g);
           } else {
             wstash_pull_fg16<S>(I, P, s, c0, c0g, r, f, g);
           }
-          wstash_pull<S, 2, true>(I, P, s, c0, c0g, r, x, h);
+          wstash_pull_h<S, FMA_C>(I, P, s, c0, r, x, h);
           g0lo = __half2float(reinterpret_cast<const __half*>(s + Fmt::LO)[c0lo]) * G0LO_INV;
         }
         mbar_arrive(ebar);  // done with the slot (the arrive orders the reads before it)
@@ -965,7 +964,8 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
       if (m <= yb + 1) {
         // moments of the column at offset dj from the own one into ring
         // entry ci of c and, if pt, of p and T
-        auto moments = [&](int dj, int cxw, int ci, bool pt) {
+        auto moments = [&](auto site, int dj, int cxw, int ci, bool pt) {
+          constexpr unsigned FMA = wall_fma<S, VAR>(site.value);
           const Phys<C> P = params();
           if (m < ny) {
             const int mr = m >= 0 ? m : -1 - m;
@@ -996,7 +996,7 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
             if (done) {
             } else if constexpr (MIX) {
               C vh[9], g0lo, clo;
-              wstash_pull_mix<true>(I, P, s, c0 + dj, mr, cxw, vf, v, vh, g0lo);
+              wstash_pull_mix<FMA>(I, P, s, c0 + dj, mr, cxw, vf, v, vh, g0lo);
               cring[ci] = moment_c(v, g0lo, clo);
               if (m < 0) cring[ci] = wet_ghost(P, cring[ci], -1 - m);
               clr[ci] = __float2half_rn(clo * G0LO_SCALE);
@@ -1021,7 +1021,7 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
               clr[ci] = __float2half_rn(clo * G0LO_SCALE);
               if (pt) {
                 pring[ci] = sum9(vf);
-                wstash_pull<S, 2, true>(I, P, s, c0 + dj, c0g + dj, mr, cxw, v);
+                wstash_pull_h<S, FMA>(I, P, s, c0 + dj, mr, cxw, v);
                 C T = dv(sum9(v), P.rho_cv, P.inv_rho_cv);
                 if (m < 0) T = ghost_T<S>(I, cxw, true, T);
                 Tring[ci] = T;
@@ -1038,9 +1038,12 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
             }
           }
         };
-        if (!helper) moments(0, xw, o2 + t + 2, true);
+        if (!helper)
+          moments(std::integral_constant<PullFor, FOR_MOMENTS>{}, 0, xw, o2 + t + 2, true);
         // the halo columns: c of all four, p and T of x0 - 1 and x0 + NC
-        if (halo) moments(hj - own, wrapx(x0 + hj, nx), o2 + hj + 2, lane == 1 || lane == 2);
+        if (halo)
+          moments(std::integral_constant<PullFor, FOR_HALO>{}, hj - own, wrapx(x0 + hj, nx),
+                  o2 + hj + 2, lane == 1 || lane == 2);
       }
       __syncthreads();
       if (s_abort) break;
@@ -1053,8 +1056,8 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
         const C* cc2 = cring + o2;
         auto normal = [&](int j) {
           C gx, gy;
-          normal3(ca, cb, cc2, j + 2, (REG ? P_reg : s_phys).eta_n2, nxr[nr(mn) + j + 2], nyr[nr(mn) + j + 2], gx,
-                  gy);
+          const int n = nr(mn) + j + 2;
+          normal3(ca, cb, cc2, j + 2, s_phys.eta_n2, nxr[n], nyr[n], gx, gy);
         };
         if (!helper) normal(t);
         // the halo columns x0 - 1 and x0 + NC
