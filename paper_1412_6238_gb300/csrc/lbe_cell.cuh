@@ -361,7 +361,12 @@ __device__ __forceinline__ Drive<S> drive(const Phys<typename S::C>& P, int gy,
 // row's) when dhc = rho c_v dT_r/dy, or already in this row's reference when
 // dhc = 0 (the wall rows); the change, w_i xi_iy dhc, enters through the
 // source term instead, (1 - omega_T) times (see below).
-template <class S, class Out>
+// DIAG: how the FP32 forms round xi_i.u/c_s^2 of the diagonal directions (fixed
+// here: left to the compiler it follows what else uses 3 u_x, and a state would
+// not go on bit for bit under the next build): 0 from the rounded 3 u_x and
+// 3 u_y; 1, 2 by a fused multiply-add, in directions 6 and 8 of 3 u_y (1) or of
+// 3 u_x (2).
+template <class S, int DIAG = 0, class Out>
 __device__ __forceinline__ void collide(const Phys<typename S::C>& P, const typename S::C f[9],
                                         const typename S::C g[9], const typename S::C h[9],
                                         typename S::C cc, typename S::C pp, typename S::C TT,
@@ -533,12 +538,14 @@ __device__ __forceinline__ void collide(const Phys<typename S::C>& P, const type
     a = uy3;
     hq = C(0.5) * (a * a - uu);
     dir2(2, 4, wa, Ka, a, hq, Jy, Jyl, Fy, Gy, wa * dhc);
-    a = ux3 + uy3;
-    hq = C(0.5) * (a * a - uu);
-    dir2(5, 7, wd, Kd, a, hq, Jp, Jpl, Fx + Fy, Gx + Gy, wd * dhc);
-    a = uy3 - ux3;
-    hq = C(0.5) * (a * a - uu);
-    dir2(6, 8, wd, Kd, a, hq, Jm, Jml, Fy - Fx, Gy - Gx, wd * dhc);
+    const C ap = DIAG == 0 ? __fadd_rn(ux3, uy3) : fmaf(C(3), ux, uy3);
+    hq = C(0.5) * (ap * ap - uu);
+    dir2(5, 7, wd, Kd, ap, hq, Jp, Jpl, Fx + Fy, Gx + Gy, wd * dhc);
+    const C am = DIAG == 0   ? __fsub_rn(uy3, ux3)
+                 : DIAG == 1 ? fmaf(C(3), uy, -ux3)
+                             : fmaf(C(-3), ux, uy3);
+    hq = C(0.5) * (am * am - uu);
+    dir2(6, 8, wd, Kd, am, hq, Jm, Jml, Fy - Fx, Gy - Gx, wd * dhc);
     const C W0 = WGT<C>(0);
     const C G0 = W0 + W0 * hu;
     // rest direction: f and hbar take minus the sum of the moving increments

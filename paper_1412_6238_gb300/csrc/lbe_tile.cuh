@@ -412,7 +412,8 @@ struct Tile {
       // the dissipation term
       C du[4] = {C(0), C(0), C(0), C(0)};
       if (I.uvel != nullptr) grad_u(nx, ny, I.uvel, gx, gy, du);
-      collide<S>(P, f, g, h, cc, pp, TT, st.gpx, st.gpy, d,
+      constexpr int DIAG = S::kind == ST_F32 && TY == 4 ? 2 : 1;  // (see collide)
+      collide<S, DIAG>(P, f, g, h, cc, pp, TT, st.gpx, st.gpy, d,
                  [&](int k, int i, C v) {
                    if constexpr (S::SR) {
                      v = S::sr_value(I, k, i, v, hc);
@@ -529,7 +530,7 @@ drive_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_tiles,
     const bool dis = I.dissip != 0;
     if (dis) grad_u(nx, ny, w + DRIVE_UX * N, x, y, du);
     C lo_out = C(0);
-    collide<S>(
+    collide<S, 1>(
         P, f, g, h, cc, p[1][1], w[DRIVE_T * N + k], gpx, gpy, d,
         [&](int l, int i, C v) { st_cell<S>(I, dst, l, i, rowbase, x, v); }, g0lo, clo, &lo_out,
         (y > 0 && y < ny - 1) ? P.dh : C(0), dis ? du : nullptr);

@@ -2,8 +2,8 @@
 the compiler's choice wherever a kernel does not fix it, and in the 16-bit
 storages a value next to a tie is then stored the other way: a run continued
 under another build would part from its own past.  The digests are of states
-made before the kernels read their constants from shared memory; inputs are
-built from whole numbers, so that no library function enters.  The wide grid is
+made before the kernels read their constants from shared memory and before the
+FP64 quotients were rewritten; inputs are built from whole numbers, so that no library function enters.  The wide grid is
 all walls and strip edges, the other one mostly bulk."""
 import hashlib
 import json
@@ -25,7 +25,7 @@ def cases():
     for storage in ("f32", "f16mix", "f16dev", "bf16dev"):
         for options in ("plain", "variants"):
             for nx, ny in GRIDS:
-                for kernel in (7, 8):
+                for kernel in (0, 1, 2, 3, 4, 7, 8):
                     yield storage, options, nx, ny, kernel
 
 
