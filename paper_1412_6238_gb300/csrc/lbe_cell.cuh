@@ -476,8 +476,9 @@ __device__ __forceinline__ void collide(const Phys<typename S::C>& P, const type
                                    __fmul2_rn(__fmul2_rn(aTiv, gd), __fmul2_rn(rT, G)));
       ho = __fadd2_rn(ho, sT);
       if (wdu) {  // the dissipation term: isotropic part whole, the rest (1 - omega_T/2)
-        ho.x += aT * (ws[i] - W * ws0) + W * ws0;
-        ho.y += aT * (ws[j] - W * ws0) + W * ws0;
+        const C iso = __fmul_rn(W, ws0);
+        ho.x += fmaf(aT, __fsub_rn(ws[i], iso), iso);
+        ho.y += fmaf(aT, __fsub_rn(ws[j], iso), iso);
       }
       // increments, whose sum the rest direction takes with the opposite sign
       dfs += finc.x + finc.y;
@@ -509,10 +510,15 @@ __device__ __forceinline__ void collide(const Phys<typename S::C>& P, const type
         const C d_i = ((Sf - f[i]) + Af) + Afl, d_j = ((Sf - f[j]) - Af) - Afl;
         const C Gi = W * (C(1) + (a + hq)), Gj = W * (C(1) + (hq - a));
         auto one = [&](int k, C G, C dl) {
-          const C ex = C(EX(k)), ey = C(EY(k));
-          const C fph = d.rho * G - C(3) * af * dl;
-          const C q = (ex - ux) * (ex * wdu[0] + ey * wdu[1]) +
-                      (ey - uy) * (ex * wdu[2] + ey * wdu[3]);
+          // (rounded as written, so that the step and the pass after a pre-pass
+          // agree bit for bit)
+          const C fph = fmaf(d.rho, G, -__fmul_rn(C(3) * af, dl));
+          auto along = [&](C dx, C dy) {  // (xi_k.grad) of a velocity component
+            const C a = EX(k) < 0 ? -dx : dx, b = EY(k) < 0 ? -dy : dy;
+            return EX(k) == 0 ? b : EY(k) == 0 ? a : __fadd_rn(a, b);
+          };
+          const C q = fmaf(C(EY(k)) - uy, along(wdu[2], wdu[3]),
+                           __fmul_rn(C(EX(k)) - ux, along(wdu[0], wdu[1])));
           ws[k] = -fph * q;
         };
         one(i, Gi, d_i);
