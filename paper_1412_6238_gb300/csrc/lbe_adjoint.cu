@@ -426,9 +426,9 @@ __device__ __forceinline__ void copy_async4(void* dst, const void* src) {
 // theta sums.
 template <class R>
 __global__ void __launch_bounds__(TPB, sizeof(R) == 4 ? 2 : 1)
-adjoint_A(Geo G, const InstDev* __restrict__ d, State<R> st, const R* __restrict__ a,
-          const R* __restrict__ at, const double* __restrict__ obs, double wl,
-          R* __restrict__ aout, R* __restrict__ S, double* __restrict__ part) {
+adjoint_A(Geo G, const InstDev* __restrict__ d, State<R> st, const R* a, const R* at,
+          const double* obs, double wl, R* __restrict__ aout, R* __restrict__ S,
+          double* __restrict__ part) {
   grid_wait();
   extern __shared__ __align__(16) char smem_raw[];
   TileA<R>& sm = *reinterpret_cast<TileA<R>*>(smem_raw);
@@ -722,7 +722,7 @@ struct TileB {
 
 template <class R>
 __global__ void __launch_bounds__(TPB)
-adjoint_B(Geo G, const InstDev* __restrict__ d, State<R> st, const R* __restrict__ S,
+adjoint_B(Geo G, const InstDev* __restrict__ d, State<R> st, const R* S,
           R* __restrict__ tout) {
   grid_wait();
   using Tl = TileB<R>;

@@ -154,7 +154,10 @@ struct StepCount {
   const uint32_t* base;
   uint32_t ahead;
 #ifdef __CUDACC__
-  __device__ __forceinline__ uint32_t now() const { return __ldg(base) + ahead; }
+  // (volatile: after grid_wait, where the kernel before may have written it)
+  __device__ __forceinline__ uint32_t now() const {
+    return *static_cast<const volatile uint32_t*>(base) + ahead;
+  }
 #endif
 };
 
@@ -290,6 +293,8 @@ __device__ __forceinline__ __nv_bfloat16 sr_bf16(float x, uint32_t r) {
 
 // ------------------------------------------------------------ storage codecs
 // ld / st take (k, i) as template-folded constants through the unrolled loops.
+// Ordinary loads: a step starts while the one before still writes (launch_early),
+// so nothing here is read-only for a kernel's whole life.
 // FP64 stores the populations as they are (parity mode).  The other forms
 // store hbar as the deviation hbar_i - w_i rho c_v T_r(y) from the linear
 // conduction profile T_r of the row the value is stored in; the kernels work
@@ -304,7 +309,7 @@ struct StF64 {
   }
   __device__ static __forceinline__ C ld(const InstDev& I, const Phys<C>&, const char* b, int k,
                                          int i, size_t idx) {
-    return __ldg(reinterpret_cast<const double*>(b + (size_t)(k * 9 + i) * I.plane_bytes) + idx);
+    return reinterpret_cast<const double*>(b + (size_t)(k * 9 + i) * I.plane_bytes)[idx];
   }
   __device__ static __forceinline__ void st(const InstDev& I, char* b, int k, int i, size_t idx,
                                             C v) {
@@ -322,8 +327,8 @@ struct StF32 {
   __device__ static __forceinline__ C ld(const InstDev& I, const Phys<C>&, const char* b, int k,
                                          int i, size_t idx) {
     if (k < 2)
-      return __ldg(reinterpret_cast<const float*>(b + (size_t)i * I.pair_bytes) + 2 * idx + k);
-    return __ldg(reinterpret_cast<const float*>(b + I.h_off + (size_t)i * I.plane_bytes) + idx);
+      return reinterpret_cast<const float*>(b + (size_t)i * I.pair_bytes)[2 * idx + k];
+    return reinterpret_cast<const float*>(b + I.h_off + (size_t)i * I.plane_bytes)[idx];
   }
   __device__ static __forceinline__ void st(const InstDev& I, char* b, int k, int i, size_t idx,
                                             C v) {
@@ -368,8 +373,7 @@ struct StDev {
   }
   __device__ static __forceinline__ C ld(const InstDev& I, const Phys<C>& P, const char* b, int k,
                                          int i, size_t idx) {
-    if (k == 1 && i == 0)
-      return __ldg(reinterpret_cast<const float*>(b + I.g0_off) + idx);
+    if (k == 1 && i == 0) return reinterpret_cast<const float*>(b + I.g0_off)[idx];
     return cvt(*at(I, b, k, i, idx)) * P.inv_s[k];
   }
   __device__ static __forceinline__ void st(const InstDev& I, char* b, int k, int i, size_t idx,
@@ -443,8 +447,8 @@ struct StMix {
   }
   __device__ static __forceinline__ C ld(const InstDev& I, const Phys<C>& P, const char* b, int k,
                                          int i, size_t idx) {
-    if (k == 0) return __ldg(reinterpret_cast<const float*>(word(I, b, i, idx)));
-    if (k == 1 && i == 0) return __ldg(reinterpret_cast<const float*>(b + I.g0_off) + idx);
+    if (k == 0) return *reinterpret_cast<const float*>(word(I, b, i, idx));
+    if (k == 1 && i == 0) return reinterpret_cast<const float*>(b + I.g0_off)[idx];
     return __half2float(*reinterpret_cast<const __half*>(word(I, b, i, idx) + half_at(k, i))) *
            P.inv_s[k];
   }

@@ -488,7 +488,7 @@ drive_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_tiles,
     char* __restrict__ dst = I.buf[parity ^ 1];
     const Phys<C> P = phys<C>(I);
     const size_t N = (size_t)nx * ny, k = (size_t)y * nx + x, rowbase = (size_t)y * I.pitch;
-    const C* __restrict__ w = static_cast<const C*>(I.drive);
+    const C* w = static_cast<const C*>(I.drive);
     const Cell<S> q = make_cell<S>(x, y, nx);
     C f[9], g[9], h[9];
     C cc = w[DRIVE_C * N + k], g0lo = C(0), clo = C(0);
@@ -515,7 +515,7 @@ drive_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_tiles,
     set_momentum<S>(d, jx, jy, jxl, jyl);
     // p of the neighbours: x wraps, the ghost rows mirror
     C p[3][3];
-    const C* __restrict__ wp = w + DRIVE_P * N;
+    const C* wp = w + DRIVE_P * N;
 #pragma unroll
     for (int j = 0; j < 3; j++) {
       const int yy = y - 1 + j;

@@ -72,7 +72,7 @@ def golden(storage, options, nx, ny, kernel):
         return json.load(f)["%s %s %dx%d kernel %d" % (storage, options, nx, ny, kernel)]
 
 
-@pytest.mark.parametrize("storage,options,nx,ny,kernel", cases())
+@pytest.mark.parametrize("storage,options,nx,ny,kernel", list(cases()))
 def test_state_bits(storage, options, nx, ny, kernel):
     assert digest(storage, options, nx, ny, kernel) == golden(storage, options, nx, ny, kernel)
 
