@@ -218,7 +218,8 @@ lbe_status lbe_load(lbe_handle* h, const char* path);
 
 /* Step-kernel choice (autotuner hook).  Kernel ids 0 .. lbe_num_tiles()-1:
  * ids whose shape has ty > 0 are the tile kernel with TX x TY cells per CTA
- * (any storage; FP64 provides id 0 only); ids 7 and 8 (ty == 0) are the
+ * (any storage; FP64 provides id 0 only, and takes a shape of its own by the
+ * size of the grids: 4 x 8 or 16 x 8); ids 7 and 8 (ty == 0) are the
  * strip kernel with 128 output columns per CTA marching over rows, staging
  * each row's pulled populations in shared memory with bulk copies (16/32-bit
  * and F16MIX storages, every instance at least 4 columns wide; the default
@@ -235,6 +236,10 @@ lbe_status lbe_load(lbe_handle* h, const char* path);
  * at most -seg_rows rows; 0: automatic (balanced ranges when the instances
  * differ in size, else items with the row count chosen from the wave
  * count, at most 96).  LBE_EINVAL for a kernel the handle cannot use.
+ * With the dissipation term or a density ratio in every instance, id 0 with
+ * grid_ctas = 0 leaves what a pass before the step computes to a pass that
+ * collides, 128 cells per CTA; any other choice runs the step that computes it
+ * again (the same state for id 0).
  * lbe_get_tile() reports {kernel id, grid CTAs, seg rows, work items}. */
 int32_t lbe_num_tiles(void);
 lbe_status lbe_tile_shape(int32_t tile_id, int32_t* tx, int32_t* ty);

@@ -29,7 +29,7 @@ struct InstHost {
   double* walls = nullptr;  // device: Tbot[nx], Ttop[nx], then 4 float tables
   double* pcorr = nullptr;  // device [ny][nx]: corrected p (varying density only)
   double* uvel = nullptr;   // device [2][ny][nx]: u of every cell (dissipation term only)
-  void* drive = nullptr;    // device: the pre-pass's planes, instead of pcorr and uvel
+  void* drive = nullptr;    // device: the pre-pass's planes; pcorr and uvel lie in them then
   std::vector<double> Tbot, Ttop;
   std::vector<float> wdev;  // host copy of the T_w - T_r tables
 };
@@ -53,6 +53,8 @@ struct lbe_handle {
   InstDev* d_pinst = nullptr;    // [n] shape-0 work list of the pcorr pass (vrho)
   int64_t p_tiles = 0;           // its tiles
   int p_grid = 0;                // its CTAs
+  bool planes = false;           // every instance holds the pre-pass's planes
+  bool use_planes = false;       // and the chosen kernel is the one that takes them
   int tile = 0;                  // kernel id
   int shape = 0;                 // tile kernel: the shape it runs (FP64: one of its own)
   int grid_req = 0;              // 0 = auto, -1 = one CTA per tile, >0 = CTAs
@@ -270,7 +272,7 @@ void fill_desc(lbe_handle* h, int j, InstDev& D) {
   P.kw = p.cos_wet * std::sqrt(2.0 * p.beta) / p.eps;
   D.pcorr = H.pcorr;
   D.uvel = H.uvel;
-  D.drive = H.drive;
+  D.drive = h->use_planes ? H.drive : nullptr;
   D.dissip = H.p.dissip;
   P.eta_n2 = p.eta_n * p.eta_n;
   // divisors: the rounded reciprocal and how a quotient is formed from it
@@ -344,6 +346,7 @@ void free_handle(lbe_handle* h) {
   for (auto& H : h->inst) {
     if (H.arena) cudaFree(H.arena);
     if (H.walls) cudaFree(H.walls);
+    if (H.drive) H.pcorr = H.uvel = nullptr;  // (parts of it)
     if (H.pcorr) cudaFree(H.pcorr);
     if (H.uvel) cudaFree(H.uvel);
     if (H.drive) cudaFree(H.drive);
@@ -403,11 +406,39 @@ void take_drive_planes(lbe_handle* h) {
       H.drive = nullptr;
       continue;
     }
-    if (H.pcorr) cudaFree(H.pcorr);
-    if (H.uvel) cudaFree(H.uvel);
-    H.pcorr = H.uvel = nullptr;
+    // another kernel's pre-pass (lbe_set_tile) finds its planes in the same memory
+    const size_t N = (size_t)H.nx * H.ny;
+    double* const at = static_cast<double*>(H.drive);
+    static_assert(DRIVE_NUM * sizeof(float) >= 3 * sizeof(double), "room for pcorr and uvel");
+    if (H.pcorr) {
+      cudaFree(H.pcorr);
+      H.pcorr = at;
+    }
+    if (H.uvel) {
+      cudaFree(H.uvel);
+      H.uvel = at + N;
+    }
     fill_desc(h, j, h->idev[j]);
   }
+  h->planes = ok;
+}
+
+// The pre-pass's work list: tiles of all instances.
+lbe_status upload_prepass(lbe_handle* h) {
+  const TileShape pre = TILE_SHAPES[pre_shape(h->storage)];
+  std::vector<InstDev> f = h->idev;
+  int64_t begin = 0;
+  for (auto& D : f) {
+    D.tiles_x = (D.nx + pre.tx - 1) / pre.tx;
+    D.tiles_y = (D.ny + pre.ty - 1) / pre.ty;
+    D.tile_begin = begin;
+    begin += (int64_t)D.tiles_x * D.tiles_y;
+  }
+  h->p_tiles = begin;
+  h->p_grid = (int)std::min<int64_t>(begin, (int64_t)4 * h->num_sms);
+  CU(h, cudaMemcpyAsync(h->d_pinst, f.data(), sizeof(InstDev) * h->n, cudaMemcpyHostToDevice,
+                        h->stream));
+  return wait(h);
 }
 
 // Rows per item of the strips (nc columns) of n instances: of lo..hi, the one
@@ -491,6 +522,15 @@ lbe_status setup_tiles(lbe_handle* h) {
     return wait(h);
   }
   h->shape = h->storage == LBE_F64 ? f64_shape(h) : h->tile;
+  // the planes are for kernel 0 as it launches itself; another one, or a grid of
+  // the caller's, computes again what they would hold
+  h->use_planes = h->planes && h->tile == 0 && h->grid_req == 0;
+  for (int j = 0; j < h->n; j++)
+    h->idev[j].drive = h->use_planes ? h->inst[j].drive : nullptr;
+  if (h->d_pinst) {
+    const lbe_status st = upload_prepass(h);
+    if (st) return st;
+  }
   const TileShape ts = TILE_SHAPES[h->shape];
   int64_t begin = 0;
   for (int j = 0; j < h->n; j++) {
@@ -511,6 +551,10 @@ lbe_status setup_tiles(lbe_handle* h) {
     h->grid = h->grid_req;
   else
     h->grid = occ * h->num_sms;
+  if (h->use_planes) {  // what drive_kernel is launched with
+    h->total_tiles = h->p_tiles * drive_parts(h->storage);
+    h->grid = (int)std::min<int64_t>(h->total_tiles, 2147483647);
+  }
   drop_graph(h);
   h->graph_failed = false;
   return wait(h);
@@ -548,9 +592,10 @@ cudaError_t launch_one_step(lbe_handle* h, int parity, int64_t ahead) {
     e = h->storage == LBE_F64
             ? pcorr_f64(h->d_pinst, h->n, h->p_tiles, parity, h->p_grid, h->stream)
             : pcorr_f32(h->d_pinst, h->n, h->p_tiles, parity, h->p_grid, h->stream);
-  if (e == cudaSuccess && h->inst[0].drive)
-    return h->storage == LBE_F64 ? drive_f64(h->d_pinst, h->n, h->p_tiles, parity, h->stream)
-                                 : drive_f32(h->d_pinst, h->n, h->p_tiles, parity, h->stream);
+  if (e == cudaSuccess && h->use_planes)
+    return h->storage == LBE_F64
+               ? drive_f64(h->d_pinst, h->n, h->total_tiles, parity, h->grid, h->stream)
+               : drive_f32(h->d_pinst, h->n, h->total_tiles, parity, h->grid, h->stream);
   if (e == cudaSuccess)
     e = launch_step(h->storage, h->shape, h->d_inst, h->n, h->total_tiles, parity, h->grid,
                     count, h->stream);
@@ -839,22 +884,7 @@ lbe_status create(int32_t n, const lbe_params* params, const lbe_init_fields* in
     }
     CUB(cudaMemcpyAsync(h->d_finst, f.data(), sizeof(InstDev) * n, cudaMemcpyHostToDevice,
                         h->stream));
-    if (h->vrho || h->dissip) {
-      // the pre-pass: tiles of all instances in one work list
-      const TileShape pre = TILE_SHAPES[pre_shape(h->storage)];
-      int64_t begin = 0;
-      for (auto& D : f) {
-        D.tiles_x = (D.nx + pre.tx - 1) / pre.tx;
-        D.tiles_y = (D.ny + pre.ty - 1) / pre.ty;
-        D.tile_begin = begin;
-        begin += (int64_t)D.tiles_x * D.tiles_y;
-      }
-      h->p_tiles = begin;
-      h->p_grid = (int)std::min<int64_t>(begin, (int64_t)4 * h->num_sms);
-      CUB(cudaMalloc(&h->d_pinst, sizeof(InstDev) * n));
-      CUB(cudaMemcpyAsync(h->d_pinst, f.data(), sizeof(InstDev) * n, cudaMemcpyHostToDevice,
-                          h->stream));
-    }
+    if (h->vrho || h->dissip) CUB(cudaMalloc(&h->d_pinst, sizeof(InstDev) * n));
     CUB(cudaStreamSynchronize(h->stream));
   }
   // initial state of each instance: the rest state of every cell (three

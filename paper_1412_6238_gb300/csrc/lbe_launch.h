@@ -48,6 +48,11 @@ constexpr TileShape TILE_SHAPES[NUM_TILES + 3] = {{32, 8},  {64, 4},  {32, 16}, 
                                                   {128, 0}, {4, 8},   {16, 8},  {4, 8}};
 // The tiles of the pre-pass (and of the pass that collides after it).
 constexpr int pre_shape(int storage) { return storage == ST_F64 ? F64_TILE : 0; }
+// CTAs of the pass that collides, per tile of the pre-pass.
+constexpr int DRIVE_THREADS = 128;
+constexpr int drive_parts(int storage) {
+  return TILE_SHAPES[pre_shape(storage)].tx * TILE_SHAPES[pre_shape(storage)].ty / DRIVE_THREADS;
+}
 inline bool is_strip(int tile) { return tile >= STRIP_FIRST && tile < NUM_TILES; }
 inline bool is_stash(int tile) { return tile == STASH_ID || tile == STASH_OWN_ID; }
 
@@ -165,9 +170,12 @@ cudaError_t pcorr_f64(const InstDev* d, int n, int64_t total, int parity, int gr
 // FP32 storage: the pre-pass of the dissipation term (u of every cell)
 cudaError_t pcorr_f32(const InstDev* d, int n, int64_t total, int parity, int grid,
                       cudaStream_t s);
-// The pass that collides, after a pre-pass into every instance's `drive`.
-cudaError_t drive_f64(const InstDev* d, int n, int64_t total, int parity, cudaStream_t s);
-cudaError_t drive_f32(const InstDev* d, int n, int64_t total, int parity, cudaStream_t s);
+// The pass that collides, after a pre-pass into every instance's `drive`: `parts`
+// (drive_parts per tile of the pre-pass) on `grid` CTAs.
+cudaError_t drive_f64(const InstDev* d, int n, int64_t parts, int parity, int grid,
+                      cudaStream_t s);
+cudaError_t drive_f32(const InstDev* d, int n, int64_t parts, int parity, int grid,
+                      cudaStream_t s);
 cudaError_t fields_f32(const InstDev* d, int64_t tiles, int parity, const FieldOut& out,
                        cudaStream_t s);
 cudaError_t fields_f16(const InstDev* d, int64_t tiles, int parity, const FieldOut& out,

@@ -88,15 +88,13 @@ cudaError_t LBE_CAT(pcorr_, LBE_SUFFIX)(const InstDev* d, int n, int64_t total, 
                                          int grid, cudaStream_t s) {
   if (grid <= 0) grid = 1;
   if ((int64_t)grid > total) grid = (int)total;
-  return launch_early(tile_kernel<LBE_ST, PRE.tx, PRE.ty, 2>, dim3(grid), PRE.tx * PRE.ty, 0, s, d, n, total, parity,
-                      FieldOut{}, StepCount{});
+  return launch_early(tile_kernel<LBE_ST, PRE.tx, PRE.ty, 2>, dim3(grid), PRE.tx * PRE.ty, 0, s, d,
+                      n, total, parity, FieldOut{}, StepCount{});
 }
-cudaError_t LBE_CAT(drive_, LBE_SUFFIX)(const InstDev* d, int n, int64_t total, int parity,
-                                         cudaStream_t s) {
-  const int64_t parts = total * (PRE.tx * PRE.ty / DRIVE_THREADS);
-  return launch_early(drive_kernel<LBE_ST, PRE.tx, PRE.ty>,
-                      dim3((unsigned)std::min<int64_t>(parts, 2147483647)), DRIVE_THREADS, 0, s, d,
-                      n, total, parity);
+cudaError_t LBE_CAT(drive_, LBE_SUFFIX)(const InstDev* d, int n, int64_t parts, int parity,
+                                         int grid, cudaStream_t s) {
+  return launch_early(drive_kernel<LBE_ST, PRE.tx, PRE.ty, DRIVE_THREADS>, dim3((unsigned)grid),
+                      DRIVE_THREADS, 0, s, d, n, parts, parity);
 }
 #endif
 

@@ -462,16 +462,15 @@ tile_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_tiles, 
 
 // The step of cells whose moments, force and u the pre-pass has left in
 // I.drive: grad p, and the collisions.  One cell a thread; nothing is shared, so
-// CTAs of DRIVE_THREADS take the tiles of the pre-pass's work list in parts.
-constexpr int DRIVE_THREADS = 128;
-template <class S, int TX, int TY>
-__global__ void __launch_bounds__(DRIVE_THREADS, S::kind == ST_F64 ? 1 : 4)
-drive_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_tiles, int parity) {
+// CTAs of THREADS take the tiles of the pre-pass's work list in parts.
+template <class S, int TX, int TY, int THREADS>
+__global__ void __launch_bounds__(THREADS, S::kind == ST_F64 ? 1 : 4)
+drive_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t parts, int parity) {
   using C = typename S::C;
   static_assert(!S::SR, "no stochastic rounding here");
-  constexpr int PARTS = TX * TY / DRIVE_THREADS, ROWS = TY / PARTS;
+  constexpr int PARTS = TX * TY / THREADS, ROWS = TY / PARTS;
   grid_wait();
-  for (int64_t t = blockIdx.x; t < PARTS * total_tiles; t += gridDim.x) {
+  for (int64_t t = blockIdx.x; t < parts; t += gridDim.x) {
     int lo = 0, hi = n_inst - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;

@@ -31,7 +31,8 @@ def cases():
                     yield storage, options, nx, ny, kernel
     for options in ("dissipation", "dissipation variants"):
         for nx, ny in GRIDS:
-            yield "f32", options, nx, ny, 0
+            for kernel in range(5):
+                yield "f32", options, nx, ny, kernel
 
 
 def digest(storage, options, nx, ny, kernel, batched=False):
