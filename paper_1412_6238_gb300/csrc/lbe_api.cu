@@ -381,23 +381,24 @@ int f64_shape(const lbe_handle* h) {
 // Planes for the pre-pass of a varying density or the dissipation term to leave
 // all it computes in, so that the pass that collides need not compute it again.
 // us a step, again / left: FP64 500 x 333 density ratio 453 / 367, dissipation
-// 490 / 413; FP32 dissipation 512 x 256 35.0 / 27.3, 1000 x 700 188 / 155; FP64
+// 490 / 413; FP32 dissipation 512 x 256 35.0 / 24.5, 1000 x 700 188 / 155; FP64
 // 128 x 128 67 / 46.  Only where every instance has a pre-pass (the others
 // would be given one), not for the split tiles, and only with room to spare: a
 // grid that barely fits keeps pcorr and uvel, and so does one whose allocation
-// fails.
+// fails.  Both ways give the same bits.
 void take_drive_planes(lbe_handle* h) {
   size_t bytes = 0, room = 0, total = 0;
-  const size_t esz = h->storage == LBE_F64 ? sizeof(double) : sizeof(float);
+  const size_t per = drive_planes(h->storage) *
+                     (h->storage == LBE_F64 ? sizeof(double) : sizeof(float));
   for (auto& H : h->inst) {
     if (!H.pcorr && !H.uvel) return;
-    bytes += esz * DRIVE_NUM * (size_t)H.nx * H.ny;
+    bytes += per * (size_t)H.nx * H.ny;
   }
   if (h->storage == LBE_F64 && f64_shape(h) == SPLIT_TILE) return;
   const size_t spare = sizeof(double) * 32 * (size_t)h->max_cells + ((size_t)256 << 20);
   bool ok = cudaMemGetInfo(&room, &total) == cudaSuccess && room >= bytes + spare;
   for (auto& H : h->inst)
-    ok = ok && cudaMalloc(&H.drive, esz * DRIVE_NUM * (size_t)H.nx * H.ny) == cudaSuccess;
+    ok = ok && cudaMalloc(&H.drive, per * (size_t)H.nx * H.ny) == cudaSuccess;
   cudaGetLastError();
   for (int j = 0; j < h->n; j++) {
     InstHost& H = h->inst[j];
@@ -409,7 +410,7 @@ void take_drive_planes(lbe_handle* h) {
     // another kernel's pre-pass (lbe_set_tile) finds its planes in the same memory
     const size_t N = (size_t)H.nx * H.ny;
     double* const at = static_cast<double*>(H.drive);
-    static_assert(DRIVE_NUM * sizeof(float) >= 3 * sizeof(double), "room for pcorr and uvel");
+    static_assert(DRIVE_NUM32 * sizeof(float) >= 3 * sizeof(double), "room for pcorr and uvel");
     if (H.pcorr) {
       cudaFree(H.pcorr);
       H.pcorr = at;

@@ -143,9 +143,11 @@ struct FieldOut {
 };
 
 // Planes of InstDev::drive: what the pre-pass of a varying density or of the
-// dissipation term leaves to the pass that collides.
-enum { DRIVE_C, DRIVE_T, DRIVE_MU, DRIVE_FX, DRIVE_FY, DRIVE_GX, DRIVE_GY, DRIVE_P, DRIVE_UX,
-       DRIVE_UY, DRIVE_NUM };
+// dissipation term leaves to the pass that collides; the last three FP64
+// only (FP32 sums c in two floats anew, and has no density ratio).
+enum { DRIVE_T, DRIVE_MU, DRIVE_FX, DRIVE_FY, DRIVE_P, DRIVE_UX, DRIVE_UY, DRIVE_NUM32,
+       DRIVE_C = DRIVE_NUM32, DRIVE_GX, DRIVE_GY, DRIVE_NUM64 };
+constexpr int drive_planes(int storage) { return storage == ST_F64 ? DRIVE_NUM64 : DRIVE_NUM32; }
 
 // The number of a step: a handle's counter in device memory (the steps before
 // the current group of launches) and the step's place in the group, so that

@@ -377,13 +377,15 @@ struct Tile {
         if (I.drive != nullptr) {
           C* const o = static_cast<C*>(I.drive) + k;
           const size_t N = (size_t)nx * ny;
-          o[DRIVE_C * N] = cc;
+          if constexpr (sizeof(C) == 8) {
+            o[DRIVE_C * N] = cc;
+            o[DRIVE_GX * N] = st.gcx;
+            o[DRIVE_GY * N] = st.gcy;
+          }
           o[DRIVE_T * N] = TT;
           o[DRIVE_MU * N] = d.mu;
           o[DRIVE_FX * N] = d.Fx;
           o[DRIVE_FY * N] = d.Fy;
-          o[DRIVE_GX * N] = st.gcx;
-          o[DRIVE_GY * N] = st.gcy;
           o[DRIVE_P * N] = pcor;
           o[DRIVE_UX * N] = d.ux;
           o[DRIVE_UY * N] = d.uy;
@@ -490,12 +492,14 @@ drive_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t parts, int p
     const C* w = static_cast<const C*>(I.drive);
     const Cell<S> q = make_cell<S>(x, y, nx);
     C f[9], g[9], h[9];
-    C cc = w[DRIVE_C * N + k], g0lo = C(0), clo = C(0);
+    C cc, g0lo = C(0), clo = C(0);
     pull9<S, 0>(I, P, src, q, f);
     pull9<S, 1>(I, P, src, q, g);
     if constexpr (S::kind != ST_F64) {
       g0lo = ld_g0lo<S>(I, src, rowbase + XG + x);
       cc = moment_c(g, g0lo, clo);
+    } else {
+      cc = w[DRIVE_C * N + k];
     }
     const bool vr = sizeof(C) == 8 && nonzero(P.drho);
     Drive<S> d;
