@@ -292,8 +292,8 @@ typedef struct {
  * dT0 and dQ0 are device pointers if on_device, else host.  The handle must
  * hold one instance.  On return the handle holds the state after the N steps
  * (steps_done advanced by N).  Device memory used during the call:
- * about 32 (k + 1) + 71 values per cell (doubles for an LBE_F64 handle, floats
- * otherwise) plus N/k raw checkpoints; it is
+ * about 27 (k + 1) + 74 doubles per cell for an LBE_F64 handle, 32 (k + 1) + 71
+ * floats otherwise, plus N/k raw checkpoints; it is
  * allocated and freed inside the call (LBE_ENOMEM if it does not fit).
  * Waits. */
 lbe_status lbe_adjoint(lbe_handle* h, const lbe_adjoint_spec* spec, double* loss,

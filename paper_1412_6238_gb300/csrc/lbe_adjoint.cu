@@ -67,8 +67,11 @@ Geo make_geo(int nx, int ny) {
   return Geo{nx, ny, (nx + TX - 1) / TX, (ny + TY - 1) / TY, (int64_t)nx * ny};
 }
 
-// A state: planes of N values: the populations Q and the moments C, P, T; in
-// FP32 also the low parts of c and T.
+// A state: planes of N values: the populations Q and, in FP32, the moments C, P,
+// T and the low parts of c and T.  FP64 states are the populations alone; the
+// moments of the one in work are in planes of their own (a segment's states are
+// most of the memory of a call, and three planes more in each would be a tenth
+// of it; forming them takes 1 % of a reverse step).
 template <class R>
 struct State {
   const R *Q, *C, *P, *T, *Cl, *Tl;
@@ -164,7 +167,7 @@ __device__ __forceinline__ float sum9_exact(const float v[9], float lo0, float& 
   return hi;
 }
 
-// The state (planes of R: 27 populations, C, P, T, in FP32 Cl and Tl) of the
+// The state (planes of R: 27 populations, in FP32 C, P, T, Cl and Tl) of the
 // buffer `parity`: the pull of every cell and its moments.
 template <class S>
 __global__ void __launch_bounds__(256)
@@ -184,11 +187,7 @@ state_kernel(Geo G, const InstDev* __restrict__ d, int parity, typename S::C* __
 #pragma unroll
     for (int i = 0; i < 9; i++) out[(int64_t)i * G.N + k] = v[i];
     R lo;
-    if constexpr (two_floats<R>()) {
-      out[28 * G.N + k] = sum9_exact(v, R(0), lo);
-    } else {
-      out[28 * G.N + k] = sum9(v);
-    }
+    if constexpr (two_floats<R>()) out[28 * G.N + k] = sum9_exact(v, R(0), lo);
     pull9<S, 1>(I, P, buf, q, v);
 #pragma unroll
     for (int i = 0; i < 9; i++) out[(int64_t)(9 + i) * G.N + k] = v[i];
@@ -196,8 +195,6 @@ state_kernel(Geo G, const InstDev* __restrict__ d, int parity, typename S::C* __
       out[27 * G.N + k] =
           sum9_exact(v, ld_g0lo<S>(I, buf, (size_t)y * I.pitch + XG + x), lo);
       out[30 * G.N + k] = lo;
-    } else {
-      out[27 * G.N + k] = sum9(v);
     }
     pull9<S, 2>(I, P, buf, q, v);
     if constexpr (two_floats<R>()) {
@@ -221,12 +218,11 @@ state_kernel(Geo G, const InstDev* __restrict__ d, int parity, typename S::C* __
     } else {
 #pragma unroll
       for (int i = 0; i < 9; i++) out[(int64_t)(18 + i) * G.N + k] = v[i];
-      out[29 * G.N + k] = sum9(v) / (P.rho * P.cv);
     }
   }
 }
 
-// C, P, T of 27 FP64 planes (a state handed in by the caller)
+// C, P, T of 27 FP64 planes (an FP64 state, or one handed in by the caller)
 __global__ void moments_kernel(Geo G, const InstDev* __restrict__ d, const double* __restrict__ Q,
                                double* __restrict__ C, double* __restrict__ Pp,
                                double* __restrict__ T) {
@@ -880,7 +876,7 @@ cudaError_t step_t(const InstDev* d, const Geo& G, const State<R>& st, const R* 
 using namespace adj;
 
 size_t adjoint_real_bytes(bool fp32) { return fp32 ? 4 : 8; }
-int64_t adjoint_state_planes(bool fp32) { return fp32 ? 32 : 30; }
+int64_t adjoint_state_planes(bool fp32) { return fp32 ? 32 : 27; }
 int64_t adjoint_vector_planes() { return 27 + 3; }
 int64_t adjoint_scratch_planes() { return S_NUM; }
 int64_t adjoint_part_doubles(int nx, int ny) {

@@ -1016,7 +1016,9 @@ lbe_status adjoint_run(lbe_handle* h, const lbe_adjoint_spec& sp, double* loss, 
   if ((st = dalloc(h, abuf, 2 * vec_b, "adjoint states"))) return st;
   // scratch planes; at the end of the sweep the FP64 results for a host copy
   const size_t host_b = on_device ? 0 : sizeof(double) * (dQ0 ? S27 : dT0 ? N : 0);
-  if ((st = dalloc(h, scr, std::max(rb * (size_t)adjoint_scratch_planes() * N, host_b), "scratch")))
+  // (FP64: and the moments of the state in work)
+  const size_t scr_b = rb * (size_t)adjoint_scratch_planes() * N;
+  if ((st = dalloc(h, scr, std::max(scr_b + (fp32 ? 0 : 3 * rb * N), host_b), "scratch")))
     return st;
   // theta sums, observables of the window, partial sums of each
   if ((st = dalloc(h, small, sizeof(double) * (size_t)(4 + 4 * W) + 2 * part_b, "reductions")))
@@ -1064,10 +1066,13 @@ lbe_status adjoint_run(lbe_handle* h, const lbe_adjoint_spec& sp, double* loss, 
     }
     for (int64_t n = n1; e == cudaSuccess && n >= n0; n--) {
       const char* Q = states.p + (size_t)(n - n0) * state_b;
-      const char* cpt = Q + rb * S27;
+      char* cpt = fp32 ? nullptr : scr.p + scr_b;
+      if (cpt)
+        e = launch_adjoint_moments(d1, nx, ny, (const double*)Q, (double*)cpt, h->stream);
       const double wl = n >= first_w ? 1.0 / (double)W : 0.0;
       double* o = n >= first_w ? obs + 4 * (n - first_w) : nullptr;
-      if (o) e = launch_observable(d1, nx, ny, fp32, Q, cpt, opart, o, h->stream);
+      if (e == cudaSuccess && o)
+        e = launch_observable(d1, nx, ny, fp32, Q, cpt, opart, o, h->stream);
       if (e == cudaSuccess)
         e = launch_adjoint_step(d1, nx, ny, fp32, Q, cpt, have_next ? a_nxt : nullptr,
                                 have_next ? terms(a_nxt) : nullptr, wl, o, a_cur, terms(a_cur),

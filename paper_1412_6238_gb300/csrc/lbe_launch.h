@@ -216,14 +216,14 @@ cudaError_t launch_seed_set(uint32_t* seed, uint32_t value, cudaStream_t s);
 // states, adjoints and scratch are FP32 (a handle whose arithmetic is), else
 // FP64; sizes in planes of nx * ny values of adjoint_real_bytes.
 size_t adjoint_real_bytes(bool fp32);
-int64_t adjoint_state_planes(bool fp32);  // a state: populations and moments
+int64_t adjoint_state_planes(bool fp32);  // a state: populations, FP32: and moments
 int64_t adjoint_vector_planes();          // an adjoint: 27 planes, then 3 terms of the cell
 int64_t adjoint_scratch_planes();
 int64_t adjoint_part_doubles(int nx, int ny);  // partial sums of the tiles
 // The state of buf[parity].
 cudaError_t launch_adjoint_state(int storage, const InstDev* d_one, int nx, int ny, int parity,
                                  void* state, cudaStream_t s);
-// c, p, T (cpt[3][N]) of a caller's 27 FP64 planes.
+// c, p, T (cpt[3][N]) of 27 FP64 planes.
 cudaError_t launch_adjoint_moments(const InstDev* d_one, int nx, int ny, const double* Q,
                                    double* cpt, cudaStream_t s);
 // out4[0..1] = sum c u_y, sum c of a state.  fp32: Q is a state; else Q the 27
