@@ -119,21 +119,20 @@ __device__ __forceinline__ void tgrad(const R* v, int k, int w, R& gx, R& gy) {
   gx = sx * R(ICS2);
   gy = sy * R(ICS2);
 }
-// The same of c = c + cl (FP32: two floats) for the unit normal, differences
-// of opposite neighbours first.
-template <class R>
-__device__ __forceinline__ void cgrad(const R* c, const R* cl, int k, int w, R& gx, R& gy) {
-  const R wa = WGT<R>(1), wd = WGT<R>(5);
-  auto diff = [&](int p, int m) -> R {
-    if constexpr (two_floats<R>())
-      return (c[k + p] - c[k + m]) + (cl[k + p] - cl[k + m]);
-    else
-      return c[k + p] - c[k + m];
-  };
-  const R d1 = diff(w + 1, -w - 1), d2 = diff(1 - w, w - 1);
-  gx = R(ICS2) * (wa * diff(1, -1) + wd * (d1 + d2));
-  gy = R(ICS2) * (wa * diff(w, -w) + wd * (d1 - d2));
+// The unit normal grad c / sqrt(|grad c|^2 + eta_n^2) at entry k of c.
+__device__ __forceinline__ void unit_normal(const double* c, int k, int w, double en2, double& nx,
+                                            double& ny) {
+  const double wa = WGT<double>(1), wd = WGT<double>(5);
+  auto diff = [&](int p, int m) { return c[k + p] - c[k + m]; };
+  const double d1 = diff(w + 1, -w - 1), d2 = diff(1 - w, w - 1);
+  const double gx = ICS2 * (wa * diff(1, -1) + wd * (d1 + d2));
+  const double gy = ICS2 * (wa * diff(w, -w) + wd * (d1 - d2));
+  const double inv = 1.0 / sqrt(gx * gx + gy * gy + en2);
+  nx = gx * inv;
+  ny = gy * inv;
 }
+// (FP32: the same rounded, in two-float arithmetic: lbe_two.cuh.  In FP64 it would
+// take half as long as the rest of kernel A.)
 template <class R>
 __device__ __forceinline__ R tlap(const R* v, int k, int w) {
   const R v0 = v[k];
@@ -201,19 +200,23 @@ state_kernel(Geo G, const InstDev* __restrict__ d, int parity, typename S::C* __
       // hbar_i = v_i + w_i rho c_v T_r(y) and T = sum v / (rho c_v) + T_r(y),
       // the row's constants as two floats
       const double Tr = I.hr0 + I.hr1 * y, hr = I.pd.rho * I.pd.cv * Tr;
-      auto add = [](double c, R x, R& lo) -> R {  // c + x rounded, and the rest
+      auto add = [](double c, R x, R xl, R& lo) -> R {  // c + x + xl rounded, and the rest
         const R ch = (R)c, cl = (R)(c - (double)ch);
         R s, e;
         two_sum(ch, x, s, e);
         R r;
-        fast_two_sum(s, e + cl, r, lo);
+        fast_two_sum(s, e + (cl + xl), r, lo);
         return r;
       };
       const double w[3] = {WGT<double>(0) * hr, WGT<double>(1) * hr, WGT<double>(5) * hr};
 #pragma unroll
       for (int i = 0; i < 9; i++)
-        out[(int64_t)(18 + i) * G.N + k] = add(w[i == 0 ? 0 : i < 5 ? 1 : 2], v[i], lo);
-      out[29 * G.N + k] = add(Tr, sum9_exact(v, R(0), lo) * P.inv_rho_cv, lo);
+        out[(int64_t)(18 + i) * G.N + k] = add(w[i == 0 ? 0 : i < 5 ? 1 : 2], v[i], R(0), lo);
+      // sum v / (rho c_v), the sum and the reciprocal as two floats
+      R sl;
+      const R sh = sum9_exact(v, R(0), sl), q = __fmul_rn(sh, P.yrcv);
+      out[29 * G.N + k] =
+          add(Tr, q, fmaf(sh, P.yrcv, -q) + (sh * P.krcv + sl * P.yrcv), lo);
       out[31 * G.N + k] = lo;
     } else {
 #pragma unroll
@@ -249,6 +252,7 @@ template <class R>
 struct TileA {
   R c[CH * CW], cl[two_floats<R>() ? CH * CW : 1];
   R p[QH * QW], T[QH * QW], nx[QH * QW], ny[QH * QW];
+  Two e;  // FP32: 144 eta_n^2
 };
 
 // T of the cell k (row y), or of the ghost row y beyond a wall from its mirror
@@ -286,15 +290,18 @@ __device__ __forceinline__ void load_tile(TileA<R>& sm, const Geo& G, const Inst
       sm.T[q] = in ? tile_T(I, G, st, k, x, y) : R(0);
     }
   }
+  if (two_floats<R>() && threadIdx.x == 0) {  // (FP64, by one warp only)
+    const double e = 144.0 * I.pd.eta_n2;
+    sm.e.h = (float)e;
+    sm.e.l = (float)(e - (double)sm.e.h);
+  }
   __syncthreads();
-  const R en2 = phys<R>(I).eta_n2;
   for (int r = threadIdx.x; r < QW * QH; r += TPB) {
     const int k = (r / QW + 1) * CW + r % QW + 1;
-    R gx, gy;
-    cgrad(sm.c, sm.cl, k, CW, gx, gy);
-    const R inv = R(1) / sqrt(gx * gx + gy * gy + en2);
-    sm.nx[r] = gx * inv;
-    sm.ny[r] = gy * inv;
+    if constexpr (two_floats<R>())
+      unit_normal(sm.c, sm.cl, k, CW, sm.e, sm.nx[r], sm.ny[r]);
+    else
+      unit_normal(sm.c, k, CW, I.pd.eta_n2, sm.nx[r], sm.ny[r]);
   }
   __syncthreads();
 }
@@ -348,11 +355,7 @@ observable_kernel(Geo G, const InstDev* __restrict__ d, State<R> st, double* __r
   __syncthreads();
   for (int r = threadIdx.x; r < QW * QH; r += TPB) {
     const int k = (r / QW + 1) * CW + r % QW + 1;
-    double gx, gy;
-    cgrad<double>(sm.c, nullptr, k, CW, gx, gy);
-    const double inv = 1.0 / sqrt(gx * gx + gy * gy + P.eta_n2);
-    sm.nx[r] = gx * inv;
-    sm.ny[r] = gy * inv;
+    unit_normal(sm.c, k, CW, P.eta_n2, sm.nx[r], sm.ny[r]);
   }
   __syncthreads();
   const int tx = threadIdx.x % TX, ty = tile_row();

@@ -328,6 +328,7 @@ void fill_desc(lbe_handle* h, int j, InstDev& D) {
   float* dstf = &F.rho;
   const int nfield = (int)(sizeof(Phys<double>) / sizeof(double));
   for (int k = 0; k < nfield; k++) dstf[k] = (float)src[k];
+  F.krcv = (float)(P.yrcv - (double)F.yrcv);
   // T_w - T_r at the first / last row and at the wall positions
   D.wdev[0] = reinterpret_cast<const float*>(H.walls + 2 * H.nx);
   D.wdev[1] = D.wdev[0] + H.nx;

@@ -6,6 +6,7 @@
 #pragma once
 
 #include "lbe_common.cuh"
+#include "lbe_two.cuh"
 
 namespace lbe {
 
@@ -99,19 +100,6 @@ __device__ __forceinline__ double sum9(const double v[9]) {
 }
 __device__ __forceinline__ float sum9(const float v[9]) {
   return (((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]))) + v[8];
-}
-
-// Error-free transformations for the two-float g_0 and c of the 16/32-bit
-// forms: a + b = s + e exactly (Knuth's two-sum; the fast variant needs
-// |a| >= |b|).
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
-}
-__device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  e = b - (s - a);
 }
 
 // c = sum g_i (Eq. 28) with g_0 = g[0] + g0lo, as hi + lo: the eight small

@@ -86,7 +86,8 @@ struct Phys {
   C wmid;
   C kw;
   // FP64: 1/b rounded, and (in the low word) how a division by b is formed
-  // (lbe_cell.cuh: Den), for b = rho c_s^2, rho, rho c_v c_s^2, rho c_v
+  // (lbe_cell.cuh: Den), for b = rho c_s^2, rho, rho c_v c_s^2, rho c_v.  FP32:
+  // yrcv + krcv is 1/(rho c_v) as two floats
   C yrcs2, krcs2, yrho, krho, yrcvcs2, krcvcs2, yrcv, krcv;
 };
 
