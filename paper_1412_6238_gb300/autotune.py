@@ -3,9 +3,10 @@
 For a handle (one instance or a batch) it times every candidate launch —
 kernel id (tile shapes and strip widths), persistent-grid size and, for the
 strip kernel, rows per work item — for a few steps each and selects the
-fastest.  Results are cached in a JSON file keyed by GPU name, storage and the
-instance shapes, so a later handle of the same layout is configured without
-timing.  Timing advances the state, so the handle is checkpointed (raw
+fastest.  Results are cached in a JSON file keyed by GPU name, storage, the
+instance shapes, the options that select other kernels and the library's build,
+so a later handle of the same layout is configured without timing; a cached
+choice that the handle refuses is searched anew.  Timing advances the state, so the handle is checkpointed (raw
 storage bytes and step counter) before the search and restored after it.
 """
 from __future__ import annotations
@@ -43,10 +44,15 @@ def _store(path: str, d: dict) -> None:
     os.replace(tmp, path)
 
 
-def cache_key(device_name: str, storage: str, shapes) -> str:
-    """Key of a layout: GPU, storage and the (ny, nx) of every instance."""
+def cache_key(device_name: str, storage: str, shapes, options=(), build: str = "") -> str:
+    """Key of a layout: GPU, storage and the (ny, nx) of every instance; the
+    options of every instance that select other kernels, if any has one
+    (``LBE.options``), and the build of the library that was timed."""
     dims = ",".join("%dx%d" % (nx, ny) for ny, nx in shapes)
-    return "%s|%s|%s" % (device_name, storage, dims)
+    key = "%s|%s|%s" % (device_name, storage, dims)
+    if any(options):
+        key += "|" + ",".join(options)
+    return key + ("|" + build if build else "")
 
 
 def candidates(storage: str, shapes, num_tiles: int, tile_shape):
@@ -86,14 +92,17 @@ def tune(sim, steps: int = 10, warmup: int = 2, use_cache: bool = True) -> dict:
 
     L = _lbe.library()
     dev = torch.cuda.get_device_name(sim.stream.device)
-    key = cache_key(dev, sim.storage, sim.shapes)
+    key = cache_key(dev, sim.storage, sim.shapes, sim.options, _lbe.library_build())
     path = cache_path()
     if use_cache:
         with _lock:
             hit = _load(path).get(key)
         if hit:
-            sim.set_tile(hit["kernel"], hit["grid"], hit["seg_rows"])
-            return dict(hit, cached=True)
+            try:
+                sim.set_tile(hit["kernel"], hit["grid"], hit["seg_rows"])
+                return dict(hit, cached=True)
+            except _lbe.LBEError:
+                pass  # not a choice of this handle: search
 
     shapes_fn = lambda k: _lbe.tile_shapes()[k]  # noqa: E731
     cands = candidates(sim.storage, sim.shapes, L.lbe_num_tiles(), shapes_fn)

@@ -8,6 +8,8 @@ be built or loaded, or CUDA is unavailable, the calls raise.
 from __future__ import annotations
 
 import ctypes
+import functools
+import hashlib
 import os
 import threading
 
@@ -112,6 +114,14 @@ def library(build: bool = True) -> ctypes.CDLL:
     return _lib
 
 
+@functools.lru_cache(maxsize=None)
+def library_build() -> str:
+    """A digest of the library file: which build a measurement is of."""
+    library()
+    with open(_build.LIB, "rb") as f:
+        return hashlib.sha256(f.read()).hexdigest()[:16]
+
+
 def tile_shapes():
     L = library()
     out = []
@@ -144,6 +154,15 @@ def make_params(params: dict, storage: str | int, check_every: int = 0) -> Param
     return p
 
 
+def _options(params: dict) -> str:
+    """The options of an instance that select other kernels: r (a density
+    ratio), v (a boundary or property variant), d (the dissipation term)."""
+    get = lambda k: float(params.get(k, 0.0))  # noqa: E731
+    return (("r" if get("rho2") not in (0.0, float(params["rho"])) else "")
+            + ("v" if get("interp") or get("wall_mid") or get("cos_wet") else "")
+            + ("d" if get("dissip") else ""))
+
+
 class LBE:
     """One handle of the library: one instance, or a batch advanced together.
 
@@ -165,6 +184,7 @@ class LBE:
         self.n = len(probs)
         self.shapes = [(int(w.params["ny"]), int(w.params["nx"])) for w in probs]
         self.storage = storage
+        self.options = [_options(w.params) for w in probs]
         self.stream = stream if stream is not None else torch.cuda.Stream()
         params = (Params * self.n)()
         inits = (InitFields * self.n)()
