@@ -13,6 +13,7 @@
 
 #include "../../include/lbe.h"
 #include "lbe_launch.h"
+#include "lbe_quot.cuh"
 
 using namespace lbe;
 
@@ -278,12 +279,7 @@ void fill_desc(lbe_handle* h, int j, InstDev& D) {
   // divisors: the rounded reciprocal and how a quotient is formed from it
   auto den = [](double b, double& y, double& k) {
     y = 1.0 / b;
-    const bool mid = b > std::ldexp(1.0, -60) && b < std::ldexp(1.0, 60);
-    const int kind = b == 1.0         ? 0
-                     : b == 1.0 / 3.0 ? 4
-                     : !mid           ? 3
-                     : std::fabs(std::fma(-b, y, 1.0)) <= std::ldexp(1.0, -54) ? 1 : 2;
-    const uint64_t bits = (uint64_t)kind;
+    const uint64_t bits = (uint64_t)constant_kind(b, y);
     memcpy(&k, &bits, sizeof k);
   };
   den(P.rcs2, P.yrcs2, P.krcs2);

@@ -6,64 +6,16 @@
 #pragma once
 
 #include "lbe_common.cuh"
+#include "lbe_quot.cuh"
 #include "lbe_two.cuh"
 
 namespace lbe {
 
-// a / b in FP64, correctly rounded (parity mode rounds like the FP64
-// reference), for a divisor b > 0 whose rounded reciprocal y = RN(1/b) is at
-// hand: Markstein's iteration (P. Markstein, IBM J. Res. Dev. 34, 1990).  If q
-// is within one unit in the last place of a/b, the remainder r = a - b q is
-// exact and RN(q + r y) = RN(a/b).  q = RN(a y) is that close where the
-// residual |1 - b y| <= 2^-54 (kind 1: 3 operations); any other y needs one
-// more iteration first (kind 2: 5).  The true division takes about 10, and a
-// cell has 55 of them on a pipe with 1/64 of the FP32 rate.  Outside
-// 2^-900 <= |a| < 2^900, where a remainder could underflow, the true division.
-static __device__ __noinline__ double div_full(double a, double b) { return a / b; }
-template <int KIND>
-__device__ __forceinline__ double div_by(double a, double b, double y) {
-  const double q0 = a * y;
-  double q = fma(fma(-b, q0, a), y, q0);
-  if (KIND == 2) q = fma(fma(-b, q, a), y, q);
-  const unsigned hi = (unsigned)__double2hiint(a);
-  if (((hi >> 20) & 0x7ffu) - 123u < 1800u) return q;
-  // zero of the right sign (q is +0 for both)
-  if (((hi << 1) | (unsigned)__double2loint(a)) == 0u) return q0;
-  return div_full(a, b);
-}
-// a / fl(1/3), correctly rounded, in 2 operations.  fl(1/3) = (1 - 2^-54)/3, so
-// the quotient is 3 a + 3 a 2^-54 (1 + 2^-54 + ...), and 3 a is a multiple of a
-// quarter of the result's last place (ulp) while the second term lies between
-// a quarter and a half of it: rounding that term to a product and adding it in
-// one fused operation could miss a rounding boundary only where it is within
-// 2^-53 of ulp/4 or ulp/2, that is for 3 a next to a power of two, where
-// divisibility by 3 excludes the cases.  (Checked against the division for
-// every mantissa within 2^30 of those places.)
-__device__ __forceinline__ double dv_cs2(double a) {
-  const double q = fma(3.0, a, a * 0x1.8p-53);
-  const unsigned hi = (unsigned)__double2hiint(a);
-  // (for a zero q is the zero of the same sign)
-  if (((hi >> 20) & 0x7ffu) < 123u && ((hi << 1) | (unsigned)__double2loint(a)) != 0u)
-    return div_full(a, 1.0 / 3.0);
-  return q;
-}
 __device__ __forceinline__ float dv_cs2(float a) { return a * 3.f; }
 // c_s^2 = 1/3 of D2Q9
 template <class C>
 __device__ __forceinline__ C cs2() { return C(1.0 / 3.0); }
 
-// A divisor b: y = 1/b (FP64: rounded) and the kind: 1, 2 as above, 0 for b =
-// 1, 4 for b = fl(1/3), 3 for the true division.
-template <class C>
-struct Den {
-  C b, y;
-  int kind;
-};
-__device__ __forceinline__ double dv(double a, const Den<double>& d) {
-  if (d.kind == 0) return a;
-  if (d.kind == 4) return dv_cs2(a);
-  return d.kind == 1 ? div_by<1>(a, d.b, d.y) : (d.kind == 2 ? div_by<2>(a, d.b, d.y) : a / d.b);
-}
 __device__ __forceinline__ float dv(float a, const Den<float>& d) { return a * d.y; }
 __device__ __forceinline__ float dv(float a, float, float inv_b) { return a * inv_b; }
 // (the kind is stored in the low word of a constant)
@@ -79,7 +31,7 @@ struct Dens {
 __device__ __forceinline__ Dens<double> make_dens(const Phys<double>& P, double rc, bool vr) {
   if (vr) {
     const double b = rc * (1.0 / 3.0), v = (rc * P.cv) * (1.0 / 3.0);
-    return Dens<double>{{b, 1.0 / b, 2}, {rc, 1.0 / rc, 2}, {v, 0.0, 3}};
+    return Dens<double>{{b, 1.0 / b, cell_kind(b)}, {rc, 1.0 / rc, cell_kind(rc)}, {v, 0.0, 3}};
   }
   return Dens<double>{make_den(P.rcs2, P.yrcs2, P.krcs2), make_den(P.rho, P.yrho, P.krho),
                       make_den(P.rcvcs2, P.yrcvcs2, P.krcvcs2)};
@@ -180,48 +132,10 @@ __device__ __forceinline__ void normal3(const C* rs, const C* rc, const C* rn, i
   ny = gy * inv;
 }
 
-// The same stencils for c = hi + lo (16/32-bit forms): hi rows in FP32, lo
-// rows as FP16 of lo * 2^24; differences of hi and of lo are taken first.
+// The low part of c (16/32-bit forms), kept as FP16 of lo * 2^24.
 __device__ __forceinline__ float lo_at(const __half* r, int x) {
   return __half2float(r[x]) * G0LO_INV;
 }
-__device__ __forceinline__ void grad3c(const float* rs, const float* rc, const float* rn,
-                                       const __half* ls, const __half* lc, const __half* ln, int x,
-                                       float& gx, float& gy) {
-  const float wa = WGT<float>(1), wd = WGT<float>(5);
-  const float dEW = (rc[x + 1] - rc[x - 1]) + (lo_at(lc, x + 1) - lo_at(lc, x - 1));
-  const float dNS = (rn[x] - rs[x]) + (lo_at(ln, x) - lo_at(ls, x));
-  const float d1 = (rn[x + 1] - rs[x - 1]) + (lo_at(ln, x + 1) - lo_at(ls, x - 1));
-  const float d2 = (rs[x + 1] - rn[x - 1]) + (lo_at(ls, x + 1) - lo_at(ln, x - 1));
-  gx = dv_cs2(wa * dEW + wd * (d1 + d2));
-  gy = dv_cs2(wa * dNS + wd * (d1 - d2));
-}
-__device__ __forceinline__ float lap3c(const float* rs, const float* rc, const float* rn,
-                                       const __half* ls, const __half* lc, const __half* ln,
-                                       int x) {
-  const float v0 = rc[x], l0 = lo_at(lc, x);
-  const float wa = WGT<float>(1), wd = WGT<float>(5);
-  auto d = [&](const float* r, const __half* l, int xx) { return (r[xx] - v0) + (lo_at(l, xx) - l0); };
-  float t = wa * d(rc, lc, x + 1);
-  t = t + wa * d(rn, ln, x);
-  t = t + wa * d(rc, lc, x - 1);
-  t = t + wa * d(rs, ls, x);
-  t = t + wd * d(rn, ln, x + 1);
-  t = t + wd * d(rn, ln, x - 1);
-  t = t + wd * d(rs, ls, x - 1);
-  t = t + wd * d(rs, ls, x + 1);
-  return dv_cs2(2.f * t);
-}
-__device__ __forceinline__ void normal3c(const float* rs, const float* rc, const float* rn,
-                                         const __half* ls, const __half* lc, const __half* ln,
-                                         int x, float en2, float& nx, float& ny) {
-  float gx, gy;
-  grad3c(rs, rc, rn, ls, lc, ln, x, gx, gy);
-  const float inv = 1.f / sqrtf(gx * gx + gy * gy + en2);
-  nx = gx * inv;
-  ny = gy * inv;
-}
-
 // Stencil results at one cell.
 template <class C>
 struct Stencils {
