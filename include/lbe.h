@@ -184,7 +184,8 @@ lbe_status lbe_init_batch(int32_t n, const lbe_params* params,
                           lbe_handle** out);
 
 /* Enqueue nsteps time steps of every instance on the handle's stream
- * (replayed from a captured CUDA graph).  Returns after enqueueing when
+ * (from 64 steps on replayed from a captured CUDA graph of sixteen; fewer, and
+ * the rest, launched one by one).  Returns after enqueueing when
  * check_every == 0; otherwise runs the FP64 NaN/Inf scan every check_every
  * steps, waits for the stream and returns LBE_ENAN if any was found. */
 lbe_status lbe_step(lbe_handle* h, int64_t nsteps);

@@ -11,7 +11,8 @@ per-cell initial temperature perturbation dT0 (T(x, 0) = T0(x) + dT0(x)).
 The forward and the reverse sweep both run inside ``lbe_adjoint``: the
 forward stores a raw checkpoint every ``ckpt_every`` steps, the reverse
 sweep recomputes each segment from its checkpoint and back-propagates
-through it in FP64.  The gradient is computed during the forward call (one
+through it, in FP64 for an "f64" problem and in FP32 for the other storages
+(parameter sums and loss in FP64).  The gradient is computed during the forward call (one
 library call for both) and scaled by the incoming gradient in backward.
 """
 from __future__ import annotations

@@ -38,15 +38,15 @@
 // adjoint is formed once, rounded to FP32 where it is used (the value the
 // FP64 sum of the parts rounds to) and exact in FP64 in the results.  FP32
 // states hold the FP64 state's values rounded to FP32, and c and T as two
-// floats (for the normals and the observable).  The theta sums and the
-// observable are FP64.
+// floats (for the normals, which are the FP64 ones rounded, and the observable).
+// The theta sums and the observable are FP64.
 //
 // What bounds it: at 256 x 512 (FP32) a state is 16 MB and a step touches 45
-// MB, which the L2 holds but for the states of a segment.  Seven kernels over
-// FP64 planes (moments, normals, permutation, pass A, reduction, B, CD with a
-// read-modify-write of all 27 planes) took 210 us a step, much of it
-// conversions between FP64 planes and FP32 arithmetic at the FP64 pipe's rate;
-// the two kernels take 36 (27 and 9).
+// MB, which the L2 holds but for the states of a segment.  The two kernels take
+// 36 us a step (27 and 9).  As seven kernels over FP64 planes (moments, normals,
+// permutation, pass A, reduction, B, CD with a read-modify-write of all 27
+// planes) it takes 210, much of it conversions between FP64 planes and FP32
+// arithmetic at the FP64 pipe's rate.
 #include <cstdio>
 
 #include "../../include/lbe.h"

@@ -377,9 +377,9 @@ int f64_shape(const lbe_handle* h) {
 
 // Planes for the pre-pass of a varying density or the dissipation term to leave
 // all it computes in, so that the pass that collides need not compute it again.
-// us a step, again / left: FP64 500 x 333 density ratio 453 / 367, dissipation
-// 490 / 413; FP32 dissipation 512 x 256 35.0 / 24.5, 1000 x 700 188 / 155; FP64
-// 128 x 128 67 / 46.  Only where every instance has a pre-pass (the others
+// us a step, again / left: FP64 500 x 333 density ratio 471 / 370, dissipation
+// 501 / 412; FP32 dissipation 512 x 256 32.1 / 23.5, 1000 x 700 171 / 133; FP64
+// 128 x 128 61 / 46.  Only where every instance has a pre-pass (the others
 // would be given one), not for the split tiles, and only with room to spare: a
 // grid that barely fits keeps pcorr and uvel, and so does one whose allocation
 // fails.  Both ways give the same bits.
@@ -683,14 +683,17 @@ lbe_status ensure_scratch(lbe_handle* h) {
 }
 
 // Cells from which the fields of a single-precision storage come from the strip
-// kernel's marching rows: 4096 x 4096 FP32 0.49 ms, by the tile kernel (which
-// pulls a ring of 2/3 of a tile's cells besides) 1.79; 2048 x 2048 F16DEV 0.17,
-// 0.48.  The tile kernel takes c of that ring as a single sum, the strip kernel
-// every c in two floats, as the step does; both are as close to the FP64 fields,
+// kernel's marching rows (the tile kernel pulls a ring of 2/3 of a tile's cells
+// besides).  Five FP32 fields, us a call by tile / strip, FP32 and F16DEV: 4096 x
+// 4096 1,790 / 490; 1408 x 1408 188 / 80, 228 / 76; 768 x 1536 118 / 59, 143 / 56;
+// 1000 x 777 90 / 55, 78 / 46; 512 x 512 40 / 33, 40 / 33; 256 x 256 28 / 30.  The
+// line is not where the strip kernel gets faster but where fields keep their
+// bits: the tile kernel takes c of its ring as a single sum, the strip kernel
+// every c in two floats, as the step does.  Both are as close to the FP64 fields,
 // but in the u of a flow that has hardly begun, which is the difference of two
 // nearly equal terms, they differ by up to 2.4e-5 of it (a planar layer of a few
-// ten thousand cells in 16 bits).  Smaller grids, whose fields take 50 us either
-// way, keep the tile kernel and with it every bit they had.
+// ten thousand cells in 16 bits).  Below the line every field is bit for bit
+// what it was before the strip kernel wrote any.
 constexpr int64_t STRIP_FIELDS_FROM = (int64_t)1 << 21;
 lbe_status compute_fields(lbe_handle* h, int j, int which_parity, const FieldOut& out) {
   const InstHost& H = h->inst[j];
@@ -929,11 +932,17 @@ lbe_status create(int32_t n, const lbe_params* params, const lbe_init_fields* in
       cells += c;
       strips += c * ((H.nx + TILE_SHAPES[STASH_ID].tx - 1) / TILE_SHAPES[STASH_ID].tx);
     }
-    // which kernel refreshes the periodic ghost columns: the step itself for
-    // narrow instances (a batch of 64 drops 128 to 768 wide, FP32: 23.3
-    // GLUPS against 23.0 with ghost_kernel, F16MIX 27.3 against 26.3),
-    // ghost_kernel for wide ones (4096^2, FP32: 24.2 against 24.0 in the
-    // step, F16MIX 27.3 against 26.9)
+    // which kernel refreshes the periodic ghost columns: the step itself (8)
+    // for narrow instances, ghost_kernel (7) for wide ones.  us a step, 7 / 8:
+    //                  FP32           F16MIX         F16DEV
+    //   96 x 64       8.9 /   7.5    8.6 /   7.1    9.4 /   7.8
+    //   512 x 1024   30.5 /  29.4   27.7 /  25.5   30.1 /  28.8
+    //   768 x 4096  134.7 / 137.1  121.0 / 119.3  137.4 / 137.6
+    //   1152 x 4096 196.7 / 203.2  176.7 / 176.6  201.3 / 203.5
+    //   4096 x 4096   667 /   688    590 /   602    673 /   694
+    //   64 drops     1500 /  1539   1339 /  1281   1526 /  1477
+    // (64 drops of 128 to 768 columns.)  One line for all storages: FP32 alone
+    // would have it at six strips
     const int stash = strips <= 8.0 * cells ? STASH_OWN_ID : STASH_ID;
     // (the dissipation term's velocity gradients: the tile kernel only)
     h->tile = (h->storage == LBE_F64 || min_nx < XG || h->dissip) ? 0 : stash;

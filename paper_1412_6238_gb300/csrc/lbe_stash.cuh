@@ -46,11 +46,11 @@
 //   barrier; 4. unit normal of row i+1 (S2).
 // Every population is read from HBM once per step.  What bounds it (GB300,
 // 2048^2): FP32 issues 65 % of its slots and moves 79 % of the copy rate's
-// bytes at 4096^2 (665 us a step; 694 before the helper warp, the constants
-// in shared memory, the rings' common row offsets and the stepped store
-// pointers), held by the dependent chain of a row; the 16-bit forms issue 73 %
-// (F16MIX 136 M warp instructions where the address arithmetic of before made
-// it 145 M: 616 -> 590 us at 4096^2, F16DEV 693 -> 672).  Every mbarrier wait is
+// bytes at 4096^2 (667 us a step; 694 without the helper warp, with the
+// constants in registers, a ring width of its own for each ring and every
+// store's address formed anew), held by the dependent chain of a row; the
+// 16-bit forms issue 73 % (F16MIX 589 us at 4096^2, F16DEV 672, BF16DEV 682;
+// with the former addresses 616 and 693, 7 % more instructions).  Every mbarrier wait is
 // bounded (poll_lim polls): on the first time-out the CTA sets *err, issues
 // no further copy, waits (bounded again) for the copies it has in flight and
 // returns.  A drain wait that also runs out means a copy that was issued has
@@ -708,7 +708,7 @@ stash_kernel(const InstDev* __restrict__ insts, int n_inst, int64_t total_items,
     yb = __shfl_sync(0xffffffffu, yb, 0);
     char* __restrict__ dst = I.buf[parity ^ 1];
     // the instance's constants, from shared memory where they are used (held
-    // in registers over the row loop they made the loop spill)
+    // in registers over the row loop they make the FP32 loop spill)
     auto params = [&]() {
       Phys<C> P = s_phys;
       if constexpr (!VAR) {  // the variants are off: known to the compiler
