@@ -294,7 +294,7 @@ __device__ __forceinline__ void wstash_pull_h(const InstDev& I, const Phys<float
 #pragma unroll
   for (int i = 0; i < 9; i++) {
     const bool wall = (EY(i) == 1 && wb) || (EY(i) == -1 && wt);
-    float v = stash_val<S>(slot, 2, i, wall ? c0 : c0 - EX(i), P);
+    float v = wall ? stash_val<S>(slot, 2, i, c0, P) : stash_val<S>(slot, 2, i, c0 - EX(i), P);
     if (wall)
       v = link_h<FMA>(v, 2.f * WGT<float>(i) * P.rho * P.cv,
                       link_T<S>(I, P, xw, i, wb ? 0 : 1, Tw));
