@@ -167,8 +167,8 @@ def kernel_source_sha() -> str:
     from paper_1412_6238_gb300 import build as _b
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_1412_6238_gb300", "csrc")
-    for f in ("lbe_common.cuh", "lbe_cell.cuh", "lbe_tile.cuh", "lbe_stash.cuh",
-              "lbe_step_inst.cuh", "lbe_step_f32.cu"):
+    for f in ("lbe_common.cuh", "lbe_quot.cuh", "lbe_two.cuh", "lbe_cell.cuh", "lbe_tile.cuh",
+              "lbe_stash.cuh", "lbe_step_inst.cuh", "lbe_step_f32.cu"):
         src = open(os.path.join(d, f), encoding="utf-8").read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
         src = re.sub(r"//[^\n]*", " ", src)

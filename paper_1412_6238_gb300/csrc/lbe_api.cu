@@ -935,14 +935,16 @@ lbe_status create(int32_t n, const lbe_params* params, const lbe_init_fields* in
     // which kernel refreshes the periodic ghost columns: the step itself (8)
     // for narrow instances, ghost_kernel (7) for wide ones.  us a step, 7 / 8:
     //                  FP32           F16MIX         F16DEV
-    //   96 x 64       8.9 /   7.5    8.6 /   7.1    9.4 /   7.8
-    //   512 x 1024   30.5 /  29.4   27.7 /  25.5   30.1 /  28.8
-    //   768 x 4096  134.7 / 137.1  121.0 / 119.3  137.4 / 137.6
-    //   1152 x 4096 196.7 / 203.2  176.7 / 176.6  201.3 / 203.5
-    //   4096 x 4096   667 /   688    590 /   602    673 /   694
-    //   64 drops     1500 /  1539   1339 /  1281   1526 /  1477
-    // (64 drops of 128 to 768 columns.)  One line for all storages: FP32 alone
-    // would have it at six strips
+    //   96 x 64       9.0 /   7.2    8.7 /   7.0    9.7 /   7.8
+    //   512 x 1024   30.5 /  27.7   27.7 /  25.4   30.1 /  28.5
+    //   768 x 4096  134.7 / 132.9  121.1 / 119.3  137.9 / 136.1
+    //   1024 x 4096 174.7 / 174.3  156.2 / 155.0  178.0 / 176.8
+    //   1152 x 4096 196.9 / 197.4  176.9 / 176.5  202.0 / 201.5
+    //   1536 x 4096 260.9 / 263.1  229.3 / 230.7  262.2 / 263.6
+    //   4096 x 4096   668 /   663    591 /   602    676 /   687
+    //   64 drops     1500 /  1501   1340 /  1280   1531 /  1461
+    // (64 drops of 128 to 768 columns.)  The two meet between 1,024 and 1,536
+    // columns in every storage
     const int stash = strips <= 8.0 * cells ? STASH_OWN_ID : STASH_ID;
     // (the dissipation term's velocity gradients: the tile kernel only)
     h->tile = (h->storage == LBE_F64 || min_nx < XG || h->dissip) ? 0 : stash;
