@@ -43,7 +43,7 @@
 //
 // What bounds it: at 256 x 512 (FP32) a state is 16 MB and a step touches 45
 // MB, which the L2 holds but for the states of a segment.  The two kernels take
-// 36 us a step (27 and 9).  As seven kernels over FP64 planes (moments, normals,
+// 35 us a step (27 and 8).  As seven kernels over FP64 planes (moments, normals,
 // permutation, pass A, reduction, B, CD with a read-modify-write of all 27
 // planes) it takes 210, much of it conversions between FP64 planes and FP32
 // arithmetic at the FP64 pipe's rate.
